@@ -514,16 +514,15 @@ int tacaw_create(tacaw_ctx** out, int32_t device, uint64_t hbm_budget_bytes) {
     uint64_t thr = UINT64_MAX;
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
   }
-  // FFT twiddle tables, FP64 on host: exp(-2 pi i j / N) at tw_offset(N) + j
-  std::vector<float2> tw(kTwiddleEntries, make_float2(0.f, 0.f));
-  std::vector<int> lengths;
-  for (int N = 2; N <= 2048; N *= 2) lengths.push_back(N);
-  for (int N : kTwiddleOtherLengths) lengths.push_back(N);
-  for (int N : lengths)
-    for (int j = 0; j < N; ++j) {
-      const double a = -2.0 * M_PI * (double)j / (double)N;
-      tw[tw_offset(N) + j] = make_float2((float)std::cos(a), (float)std::sin(a));
-    }
+  // twiddle tables of the FFT passes, FP64 on host
+  std::vector<float2> tw(pass_total(), make_float2(0.f, 0.f));
+  for (const FftPass& q : kFftPasses)
+    for (int k = 0; k < q.ns; ++k)
+      for (int i = 1; i < q.r; ++i) {
+        const double a = -2.0 * M_PI * (double)(i * k) / (double)(q.ns * q.r);
+        const size_t at = q.r == 2 ? k : 2 * ((size_t)((i - 1) / 2) * q.ns + k) + (i - 1) % 2;
+        tw[pass_offset(q.r, q.ns) + at] = make_float2((float)std::cos(a), (float)std::sin(a));
+      }
   if (owned_alloc(ctx, &ctx->tw, tw.size()) != TACAW_OK ||
       cudaMemcpy(ctx->tw, tw.data(), sizeof(float2) * tw.size(), cudaMemcpyHostToDevice) != cudaSuccess ||
       owned_alloc(ctx, &ctx->d_status, 1) != TACAW_OK || cudaMemset(ctx->d_status, 0, sizeof(int)) != cudaSuccess ||

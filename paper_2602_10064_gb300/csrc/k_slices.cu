@@ -539,7 +539,7 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = acc[g * NX + t + T * e];
   __syncthreads();  // the FFT scratch of one group overlaps the accumulators of the next
-  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw + tw_offset(NX),
+  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   store_row<NX, MB>(v, Bp + ((size_t)bidx * ny + y0 + g) * b.Wp, b, t);
 }
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
   const int c = threadIdx.x % C, t = threadIdx.x / C, cc = blockIdx.x * C + c;
   const ColIdx<C, CC::SH> idx{c};
   const BlockSync sync;
-  const float2* tw = geo.tw + tw_offset(NY);
+  const float2* tw = geo.tw;
   if constexpr (ONE) {
     // one species pair: no accumulator held across the transforms
     const float2* src = Bp + (size_t)fs * NY * Wp + cc;
@@ -613,7 +613,7 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
   const auto sync = group_sync<T>(g);
   float2 v[E];
   load_row<NX, MB>(v, Ap + ((size_t)fs * ny + y) * b.Wp, b, t);
-  fft<NX, +1, PL>(v, sm, idx, t, geo.tw + tw_offset(NX), sync);
+  fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
   const size_t row = ((size_t)fs * ny + y) * NX;
   if (mode == 0) {
 #pragma unroll
@@ -631,7 +631,7 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
     for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
     return;
   }
-  fft<NX, -1, PL>(v, sm, idx, t, geo.tw + tw_offset(NX), sync);
+  fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
   store_row<NX, MB>(v, out + ((size_t)fs * ny + y) * b.Wp, b, t);
 }
 
@@ -662,7 +662,7 @@ __global__ void __launch_bounds__(RowVtCfg<NX>::THREADS, minb_of<K_ROW_VT, NX, R
     for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
     return;
   }
-  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw + tw_offset(NX),
+  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   store_row_compact<NX>(v, out + ((size_t)fs * ny + y) * b.Wp, b, t);
 }
@@ -682,7 +682,7 @@ __global__ void __launch_bounds__(ColTCfg<NY>::THREADS, minb_of<K_COL_T, NY, Col
   const int c = threadIdx.x % C, t = threadIdx.x / C, cc = blockIdx.x * C + c;
   const ColIdx<C, CC::SH> idx{c};
   const BlockSync sync;
-  const float2* tw = geo.tw + tw_offset(NY);
+  const float2* tw = geo.tw;
   const float2* src = Bt + (size_t)fs * NY * Wp + cc;
   float2 v[E];
 #pragma unroll
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, N
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
   float2 v[E];
   load_row_compact<NX>(v, At + ((size_t)fs * ny + y) * b.Wp, b, t);
-  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw + tw_offset(NX),
+  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   float2* dst = tout + ((size_t)fs * ny + y) * NX;
 #pragma unroll
@@ -744,7 +744,7 @@ __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL,
     v[e] = (abs(n) <= nb) ? amp * cmul(exv, ey[(size_t)p * NY + row]) : make_float2(0.f, 0.f);
     if (chi && abs(n) <= nb) v[e] = cmul(v[e], chi[(size_t)row * ap.Wp + cc]);
   }
-  fft<NY, +1, PL>(v, sm, ColIdx<C, CC::SH>{c}, t, geo.tw + tw_offset(NY), BlockSync{});
+  fft<NY, +1, PL>(v, sm, ColIdx<C, CC::SH>{c}, t, geo.tw, BlockSync{});
   float2* dst = Bpr + (size_t)p * NY * ap.Wp + cc;
 #pragma unroll
   for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * ap.Wp] = v[e];
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW,
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
   float2 v[E];
   load_row_compact<NX>(v, Bpr + ((size_t)p * ny + y) * ap.Wp, ap, t);
-  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw + tw_offset(NX),
+  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   float2* dst = psi0 + ((size_t)p * ny + y) * NX;
 #pragma unroll
@@ -820,7 +820,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
   float2* tst = reinterpret_cast<float2*>(smraw + SliceRowCfg<NX>::SMEM) + g * NX;
   if (TF) {
     load_row<NX, MB>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
-    fft<NX, +1, PL>(v, sm, idx, t, geo.tw + tw_offset(NX), sync);
+    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
 #pragma unroll
     for (int e = 0; e < E; ++e) tst[t + T * e] = v[e];
   } else {
@@ -841,12 +841,12 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
     }
   } else {
     load_row<NX, MB>(v, Apsi + ((size_t)w * ny + y) * b.Wp, b, t);
-    fft<NX, +1, PL>(v, sm, idx, t, geo.tw + tw_offset(NX), sync);
+    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
     if (!TF) cp_async_wait_all();
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = cmul(v[e], tst[t + T * e]);
   }
-  fft<NX, -1, PL>(v, sm, idx, t, geo.tw + tw_offset(NX), sync);
+  fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
   store_row<NX, MB>(v, Bpsi + ((size_t)w * ny + y) * b.Wp, b, t);
 }
 
@@ -868,7 +868,7 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
   const int c = threadIdx.x % C, t = threadIdx.x / C, cc = blockIdx.x * C + c;
   const ColIdx<C, CC::SH> idx{c};
   const BlockSync sync;
-  const float2* tw = geo.tw + tw_offset(NY);
+  const float2* tw = geo.tw;
   const float2* src = Bpsi + (size_t)w * NY * Wp + cc;
   float2 v[E];
 #pragma unroll

@@ -17,26 +17,44 @@ struct Band {
   const int* colnb;
 };
 
-// Grid shape plus the FFT twiddle tables (table for length N starts at tw + N).
+// Grid shape plus the FFT twiddle tables.
 struct Geo {
   int nx, ny;
-  const float2* tw;  // the context's twiddle tables: length n at tw + tw_offset(n)
+  const float2* tw;  // the context's twiddle tables: a pass's at tw + pass_offset(r, ns)
 };
 
-// Layout of the context's twiddle table: exp(-2 pi i j / n), j < n, at [tw_offset(n),
-// tw_offset(n) + n): the powers of two 2 .. 2048 at offset n (packed into [2, 4096)), then the
-// lengths with a factor 3 one after the other.
-__host__ __device__ constexpr int tw_offset(int n) {
-  return (n & (n - 1)) == 0 ? n
-         : n == 96          ? 4096
-         : n == 192         ? 4096 + 96
-         : n == 384         ? 4096 + 288
-         : n == 768         ? 4096 + 672
-         : n == 1152        ? 4096 + 1440
-                            : -1;
+// Twiddle tables of the FFT passes.  A pass of radix r after earlier radices of product ns
+// multiplies input i of butterfly k (k < ns) by exp(-2 pi i (i k) / (ns r)); its table holds these
+// as [pair p of i][k][2] with i = 2 p + 1, 2 p + 2 (radix 2: [k], i = 1), so that the threads of a
+// warp, which hold consecutive k, load consecutive entries.
+struct FftPass {
+  int r, ns;
+};
+constexpr FftPass kFftPasses[] = {
+    {4, 8},   {8, 8},    {4, 32},   {8, 32},  {16, 32}, {32, 32}, {4, 64},  {8, 64}, {4, 256}, {8, 16},  {16, 16},
+    {16, 64}, {2, 256},  {8, 256},  {4, 12},  {2, 48},  {4, 48},  {2, 192}, {4, 24}, {8, 96},  {6, 24},  {8, 144}};
+// Entries (float2) of the table of a pass.
+constexpr int pass_entries(int r, int ns) { return r == 2 ? ns : 2 * (r / 2) * ns; }
+// Start of its table, in float2 (all sizes are even: the pairs are 16-byte aligned); -1: no such pass.
+constexpr int pass_offset(int r, int ns) {
+  int at = 0;
+  for (const FftPass& q : kFftPasses) {
+    if (q.r == r && q.ns == ns) return at;
+    at += pass_entries(q.r, q.ns);
+  }
+  return -1;
 }
-constexpr int kTwiddleEntries = 4096 + 2592;
-constexpr int kTwiddleOtherLengths[5] = {96, 192, 384, 768, 1152};
+// The same as a constant for device code.
+template <int R, int NS>
+struct PassTable {
+  static constexpr int offset = pass_offset(R, NS);
+  static_assert(offset >= 0 && offset % 2 == 0, "pass missing from kFftPasses");
+};
+constexpr int pass_total() {
+  int at = 0;
+  for (const FftPass& q : kFftPasses) at += pass_entries(q.r, q.ns);
+  return at;
+}
 
 // One atom after binning, in the order of its slice list.  ix0/iy0 = floor of the grid
 // coordinate (x wrapped into [0, Lx), times nx / Lx, in FP64), fx/fy the remainder.
