@@ -724,7 +724,7 @@ int trans_bufs(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, int64_t nfs, 
 int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const float2* Ap, const float* V, int nfs,
                       float2* t, Scratch& sc, const TransBufs& tb, bool compact = false) {
   const Geo geo{p.nx, p.ny, ctx->tw};
-  const float sig = (float)sigma_per_VA(p.voltage_ev);
+  const float sig = (float)(sigma_per_VA(p.voltage_ev) / M_PI);  // sincospi takes units of pi
   const int bl = p.bandlimit_transmission && p.bandlimit > 0.0;
   const double W8 = (double)g->band.W * 8.0, row = (double)nfs * p.ny, fx = 5.0 * p.nx * std::log2((double)p.nx),
                fy = 5.0 * p.ny * std::log2((double)p.ny);

@@ -174,6 +174,7 @@ cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, c
                              cudaStream_t st);
 cudaError_t launch_col_pot(const Geo& g, const Band& b, const float2* Bp, const float2* mtab, int npair, int nfs,
                            float2* Ap, int static_band, cudaStream_t st);
+// sigma_pi: the interaction parameter over pi.
 // mode 0: store V; mode 1: t = exp(i sigma V), band-limit pass input (FFT_x, compact);
 // mode 2: t = exp(i sigma V) stored directly (no transmission band limit).
 cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, int nfs, int mode, float sigma,
