@@ -48,7 +48,9 @@ extern "C" {
 #define TACAW_ENOTFOUND (-7) /* unknown ticket */
 
 /* Time-transform arithmetic (tacaw_spectrum, tacaw_run). */
-#define TACAW_DFT_FP32 0   /* FP32 SIMT dense DFT: the plain path */
+/* Up to 2048 frames the first three run as an FP32 FFT, at least as accurate as any of them; the
+ * arithmetic given here is that of longer trajectories. */
+#define TACAW_DFT_FP32 0   /* FP32 SIMT dense DFT */
 #define TACAW_DFT_BF16X3 1 /* tcgen05 BF16 GEMM, hi*hi + hi*lo + lo*hi, FP32 accumulation */
 #define TACAW_DFT_TF32X3 2 /* tcgen05 TF32 GEMM, same three-product split */
 #define TACAW_DFT_BF16 3   /* tcgen05 BF16 GEMM, single product (precision study only) */

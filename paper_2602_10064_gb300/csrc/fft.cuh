@@ -1,5 +1,5 @@
-// Device FFT engine for the slice kernels (lengths: powers of two 32 .. 2048, 3 * 2^k for 96 ..
-// 768, and 1152).
+// Device FFT engine of the slice kernels and the time transform (lengths: powers of two 32 .. 4096,
+// 3 * 2^k for 96 .. 768, and 1152).
 //
 // Every 2D transform of the hot path (potential, transmission band limit, the slice step of
 // the multislice chain in Methods "Multislice Propagation") is split into 1D transforms along
@@ -452,6 +452,10 @@ __device__ __forceinline__ void fft(float2 (&v)[E], float2* sm, const Idx& idx, 
     fft_pass<2048, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<2048, E, 16, 16, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<2048, E, 8, 256, SIGN, true>(v, sm, idx, t, tw, sync);
+  } else if constexpr (N == 4096) {
+    fft_pass<4096, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<4096, E, 16, 16, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<4096, E, 16, 256, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (E == 12 && N == 96) {
     fft_pass<96, E, 12, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<96, E, 4, 12, SIGN, false>(v, sm, idx, t, tw, sync);

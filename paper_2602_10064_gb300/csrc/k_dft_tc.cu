@@ -1,5 +1,6 @@
 // Tensor-core time transform (Methods, "Workflow Architecture": psi~(k, w) = F_t[psi - <psi>_t],
-// I = |psi~|^2) as a dense real GEMM on the 5th-generation tensor cores (tcgen05).
+// I = |psi~|^2) as a dense real GEMM on the 5th-generation tensor cores (tcgen05): the single-product
+// requests, and the split ones of trajectories too long for the FFT of k_time_fft.cu.
 //
 // With W = exp(-2 pi i w n / F) = cos - i sin and the residual r_n = psi_n - <psi> (formed exactly
 // from the FP64-class mean), the complex sum becomes the real product D = A B^T:
@@ -439,18 +440,6 @@ __global__ void __launch_bounds__(256) k_mean_residual_split(const float2* __res
   }
 }
 
-// Spectrum image from the detector partial sums: SI[p][w] = sum over the tpp tiles of probe p of
-// part[tile][w], in FP64 and in tile order, rounded to float.
-__global__ void k_detector_tiles(const double* __restrict__ part, int64_t P, int64_t F, int64_t tpp,
-                                 float* __restrict__ SI) {
-  const int64_t w = blockIdx.x * (int64_t)blockDim.x + threadIdx.x, p = blockIdx.y;
-  if (w >= F || p >= P) return;
-  const double* col = part + (size_t)p * tpp * F + w;
-  double s = 0.0;
-  for (int64_t t = 0; t < tpp; ++t) s += col[(size_t)t * F];
-  SI[(size_t)p * F + w] = (float)s;
-}
-
 // Self-test of the bounded wait: one thread waits on an mbarrier that nothing ever arrives on,
 // with a short limit, so the wait runs out, sets the status word and returns (no copy or MMA
 // is in flight, no TMEM is held).
@@ -647,9 +636,8 @@ int spectrum_tc(tacaw_ctx* ctx, const float2* psi_k, int64_t P, int64_t F, const
   if (det) {
     ProfScope ps(ctx, "detector_tiles", sc.st, (double)ntiles * F * 8 + (double)P * F * 4, (double)ntiles * F);
     if (P > 65535) return set_err(ctx, TACAW_EINVAL, "too many probes");
-    k_detector_tiles<<<dim3((unsigned)((F + 127) / 128), (unsigned)P), 128, 0, sc.st>>>(part, P, F, cpp / TC_BN, S);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return cuda_err(ctx, e, "k_detector_tiles");
+    e = launch_detector_parts(part, P, F, cpp / TC_BN, S, sc.st);
+    if (e != cudaSuccess) return cuda_err(ctx, e, "k_detector_parts");
   }
   return TACAW_OK;
 }

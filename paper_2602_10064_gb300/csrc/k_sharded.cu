@@ -157,6 +157,10 @@ int tacaw_spectrum_partial(tacaw_ctx* ctx, const float* psi_k, int64_t P, int64_
   const int64_t nsel = q_sel ? n_sel : nq;
   cudaStream_t st = (cudaStream_t)stream;
   Scratch sc(st);
+  bool chirp;
+  if (time_fft_length(F, &chirp))
+    return partial_fft(ctx, reinterpret_cast<const float2*>(psi_k), reinterpret_cast<const float2*>(psi_ref), P, nf, f0,
+                       F, nq, q_sel, nsel, reinterpret_cast<float2*>(psi_tilde), st);
   float2* r;
   e = sc.get(&r, (size_t)P * nf * nsel);
   if (e != cudaSuccess) return cuda_err(ctx, e, "partial residual");

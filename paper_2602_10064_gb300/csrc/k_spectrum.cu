@@ -1,8 +1,9 @@
 // Time transform (Methods, "Workflow Architecture"):
 //   psi~(k, w) = F_t[psi(k, t) - <psi(k, t)>_t],  I(k, w) = |psi~(k, w)|^2.
 // The mean over frames and the residual are formed to FP64-class precision (the elastic part
-// is large and the inelastic signal is a small difference), as FP32 pairs.  This file holds the plain FP32 SIMT dense DFT;
-// the tensor-core variants are in k_dft_tc.cu.
+// is large and the inelastic signal is a small difference), as FP32 pairs.  This file holds the plain
+// FP32 SIMT dense DFT, of trajectories of more than 2048 frames and of tacaw_spectrum_static; the
+// tensor-core variants are in k_dft_tc.cu, the FFT of shorter trajectories in k_time_fft.cu.
 #include <cuda_runtime.h>
 
 #include "tacaw_internal.cuh"
@@ -139,6 +140,34 @@ cudaError_t launch_dft_fp32(const float2* r, const float2* twF, int64_t P, int64
   if (P > 65535 || (F + DFT_BM - 1) / DFT_BM > 65535) return cudaErrorInvalidValue;
   const dim3 grid((unsigned)((nsel + DFT_BN - 1) / DFT_BN), (unsigned)((F + DFT_BM - 1) / DFT_BM), (unsigned)P);
   k_dft_fp32<<<grid, 256, 0, st>>>(r, twF, F, nsel, nq, qsel, S);
+  return cudaGetLastError();
+}
+
+// Spectrum image from partial sums: SI[p][m] = sum over i of part[p][i][m], in FP64: 8 threads a bin
+// add every eighth part in order, then the 8 sums in order.  One thread a bin walked all parts
+// alone, 41 us at 32 probes x 256 frames x 84 parts.
+constexpr int DP_BINS = 32, DP_GROUPS = 8;
+__global__ void __launch_bounds__(DP_BINS * DP_GROUPS)
+    k_detector_parts(const double* __restrict__ part, int64_t F, int64_t nparts, float* __restrict__ SI) {
+  __shared__ double red[DP_GROUPS][DP_BINS];
+  const int b = threadIdx.x % DP_BINS, g = threadIdx.x / DP_BINS;
+  const int64_t m = blockIdx.x * (int64_t)DP_BINS + b, p = blockIdx.y;
+  double s = 0.0;
+  if (m < F)
+    for (int64_t i = g; i < nparts; i += DP_GROUPS) s += part[((size_t)p * nparts + i) * F + m];
+  red[g][b] = s;
+  __syncthreads();
+  if (g == 0 && m < F) {
+    for (int k = 1; k < DP_GROUPS; ++k) s += red[k][b];
+    SI[(size_t)p * F + m] = (float)s;
+  }
+}
+
+cudaError_t launch_detector_parts(const double* part, int64_t P, int64_t F, int64_t nparts, float* SI,
+                                  cudaStream_t st) {
+  if (P > 65535) return cudaErrorInvalidValue;
+  k_detector_parts<<<dim3((unsigned)((F + DP_BINS - 1) / DP_BINS), (unsigned)P), DP_BINS * DP_GROUPS, 0, st>>>(
+      part, F, nparts, SI);
   return cudaGetLastError();
 }
 

@@ -1,0 +1,346 @@
+// Time transform by FFT (Methods, "Workflow Architecture": psi~(k, w) = F_t[psi(k, t) - <psi(k, t)>_t],
+// I(k, w) = |psi~|^2) in one pass over the exit-wave stack, in FP32.
+//
+// A CTA takes C neighbouring q columns of one probe and all F frames: it loads them once (T threads
+// a column, E frames a thread, the engine of fft.cuh), removes the mean, transforms along the frames
+// through shared memory and stores |psi~|^2, or its sum over the columns (the spectrum image), or
+// psi~ itself (one process's share of a frame-sharded transform).  The stack is read once and the
+// result written once; the dense forms of the transform read it two or three times, write a
+// residual or split operands and do O(F) work per element where this does O(log F).  1024 frames x
+// 65536 q: 14.6 ms dense FP32, 0.31 ms here (2.5 TB/s; the loads of a CTA do not overlap its own
+// transform); a partial transform of 256 of 512 frames: 2.04 ms, 0.16 ms.
+//
+// Mean: every frame is first referred to the column's first frame, r1_n = psi_n - psi_0, which
+// rounds at the scale of the fluctuation (the difference of two nearly equal floats is exact), then
+// the mean of r1 is subtracted.  What the large static part could cost in precision is gone in the
+// first step, so both sums are plain FP32; columns that do not change give exactly zero.
+//
+// Frame counts: the engine's own lengths directly; any other F up to 2048 by Bluestein's chirp-z
+// identity m n = (m^2 + n^2 - (m - n)^2) / 2, as a cyclic convolution of length M >= 2 F - 1 with a
+// precomputed chirp spectrum (two transforms of length M; the final chirp has modulus 1 and is left
+// out where only |psi~|^2 is wanted).
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cmath>
+
+#include "fft.cuh"
+#include "tacaw_api_internal.h"
+
+namespace tacaw {
+
+// Elements per thread and columns per CTA of each length: 8 columns are 64-byte lines of the stack,
+// 16 or 32 whole lines; more columns of the long transforms would leave one CTA per SM.
+template <int N>
+struct TimeCfg {
+  static constexpr int E = N <= 64 ? 8 : (N == 768 || N == 1152) ? 24 : fft_pow2(N) ? (N >= 2048 ? 32 : 16) : 12;
+  static constexpr int T = N / E;
+  static constexpr int C = N <= 128 ? 32 : N <= 512 ? 16 : N <= 2048 ? 8 : 4;
+  static constexpr int THREADS = T * C;
+  static constexpr int SMEM = N * C * (int)sizeof(float2);
+  static constexpr int MINB = E >= 24 ? 1 : (512 / THREADS < 1 ? 1 : 512 / THREADS);
+};
+
+enum TimeOut { TIME_S, TIME_DETECTOR, TIME_TILDE };
+
+struct TimeArgs {
+  const float2* psi;  // [P][nf][in_nq]
+  const float2* ref;  // TIME_TILDE: [P][in_nq] static reference; else unused
+  int64_t P, F, nf, f0;
+  int64_t in_nq;
+  const int32_t* in_qsel;
+  int64_t nsel;
+  int64_t out_nq;
+  const int32_t* out_qsel;
+  float* S;        // TIME_S: [P][F][out_nq]
+  double* part;    // TIME_DETECTOR: [P][gridDim.x][F]
+  float2* tilde;   // TIME_TILDE: [P][F][nsel]
+  const float2* tw;     // FFT pass tables
+  const float2* chirp;  // Bluestein: exp(-i pi n^2 / F), n < F
+  const float2* bhat;   // Bluestein: spectrum of the conjugate chirp over M
+};
+
+// Column tiles one CTA of the spectrum image adds up before it stores its partial sums.  Fixed, so
+// that the order of the sums does not depend on how many probes a call holds.
+constexpr int TIME_DET_TILES = 8;
+
+template <int N, int OUT, bool BLUE>
+__global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_fft(const TimeArgs a) {
+  using TC = TimeCfg<N>;
+  constexpr int E = TC::E, T = TC::T, C = TC::C, WARPS = TC::THREADS / 32;
+  extern __shared__ __align__(16) unsigned char smraw[];
+  float2* sm = reinterpret_cast<float2*>(smraw);
+  const int64_t p = blockIdx.y + (int64_t)gridDim.y * blockIdx.z;
+  if (p >= a.P) return;
+  const int c = threadIdx.x % C, t = threadIdx.x / C;
+  const ColIdx<C, 0> idx{c};
+  const BlockSync sync;
+  const int F = (int)a.F;
+  const int64_t ntiles = (a.nsel + C - 1) / C;
+  float hi[OUT == TIME_DETECTOR ? E : 1], lo[OUT == TIME_DETECTOR ? E : 1];
+  if constexpr (OUT == TIME_DETECTOR) {
+#pragma unroll
+    for (int e = 0; e < E; ++e) hi[e] = lo[e] = 0.f;
+  }
+  const int64_t tile0 = OUT == TIME_DETECTOR ? (int64_t)blockIdx.x * TIME_DET_TILES : blockIdx.x;
+  const int64_t tile1 = OUT == TIME_DETECTOR ? (tile0 + TIME_DET_TILES < ntiles ? tile0 + TIME_DET_TILES : ntiles)
+                                             : tile0 + 1;
+  for (int64_t tile = tile0; tile < tile1; ++tile) {
+    const int64_t j = tile * C + c;
+    const bool live = j < a.nsel;
+    const int64_t jj = live ? j : a.nsel - 1;  // columns past the end repeat the last one, unstored
+    const int64_t q = a.in_qsel ? a.in_qsel[jj] : jj;
+    float2 v[E];
+    if constexpr (OUT == TIME_TILDE) {
+      const float2* col = a.psi + (size_t)p * a.nf * a.in_nq + q;
+      const float2 x0 = a.ref[(size_t)p * a.in_nq + q];
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int64_t n = t + T * e - a.f0;
+        v[e] = n >= 0 && n < a.nf ? col[(size_t)n * a.in_nq] - x0 : make_float2(0.f, 0.f);
+      }
+    } else {
+      const float2* col = a.psi + (size_t)p * F * a.in_nq + q;
+      const float2 x0 = col[0];
+      float2 sum = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int n = t + T * e;
+        v[e] = !BLUE || n < F ? col[(size_t)n * a.in_nq] : x0;
+      }
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        v[e] = v[e] - x0;
+        sum = sum + v[e];
+      }
+      // the column's sum: over the lanes of a warp that share it, then over the warps
+#pragma unroll
+      for (int o = C; o < 32; o <<= 1) {
+        sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
+        sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
+      }
+      __syncthreads();  // the previous tile's readers of the scratch are done
+      if ((threadIdx.x & 31) < C) sm[(threadIdx.x >> 5) * C + c] = sum;
+      __syncthreads();
+      sum = make_float2(0.f, 0.f);
+#pragma unroll
+      for (int w = 0; w < WARPS; ++w) sum = sum + sm[w * C + c];
+      const float inv = 1.f / (float)F;
+      const float2 mean = make_float2(sum.x * inv, sum.y * inv);
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = !BLUE || t + T * e < F ? v[e] - mean : make_float2(0.f, 0.f);
+    }
+    if constexpr (BLUE) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) {
+        const int n = t + T * e;
+        if (n < F) v[e] = cmul(v[e], __ldg(a.chirp + n));
+      }
+      fft<N, -1>(v, sm, idx, t, a.tw, sync);
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = cmul(v[e], __ldg(a.bhat + t + T * e));
+      fft<N, +1>(v, sm, idx, t, a.tw, sync);
+    } else {
+      fft<N, -1>(v, sm, idx, t, a.tw, sync);
+    }
+    if constexpr (OUT == TIME_DETECTOR) {
+      if (live) {
+#pragma unroll
+        for (int e = 0; e < E; ++e) pair_add(hi[e], lo[e], v[e].x * v[e].x + v[e].y * v[e].y);
+      }
+    } else if (live) {
+      if constexpr (OUT == TIME_S) {
+        float* dst = a.S + (size_t)p * F * a.out_nq + (a.out_qsel ? a.out_qsel[j] : j);
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int m = t + T * e;
+          if (!BLUE || m < F) dst[(size_t)m * a.out_nq] = v[e].x * v[e].x + v[e].y * v[e].y;
+        }
+      } else {
+        float2* dst = a.tilde + (size_t)p * F * a.nsel + j;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+          const int m = t + T * e;
+          if (!BLUE) dst[(size_t)m * a.nsel] = v[e];
+          else if (m < F) dst[(size_t)m * a.nsel] = cmul(v[e], __ldg(a.chirp + m));
+        }
+      }
+    }
+  }
+  if constexpr (OUT == TIME_DETECTOR) {
+    // over the columns, in FP64 and in an order fixed per bin
+    double* red = reinterpret_cast<double*>(smraw);  // [N][C]
+    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < E; ++e) red[(t + T * e) * C + c] = (double)hi[e] + (double)lo[e];
+    __syncthreads();
+    for (int m = threadIdx.x; m < F; m += TC::THREADS) {
+      double s = 0.0;
+#pragma unroll
+      for (int k = 0; k < C; ++k) s += red[m * C + (k + m) % C];
+      a.part[((size_t)p * gridDim.x + blockIdx.x) * F + m] = s;
+    }
+  }
+}
+
+// Lengths with a kernel.
+constexpr int kTimeLengths[] = {32, 64, 96, 128, 192, 256, 384, 512, 768, 1024, 1152, 2048, 4096};
+
+int time_fft_length(int64_t F, bool* chirp) {
+  for (int n : kTimeLengths)
+    if (n == F && n <= 2048) {
+      *chirp = false;
+      return n;
+    }
+  *chirp = true;
+  for (int n : kTimeLengths)
+    if (fft_pow2(n) && n >= 2 * F - 1) return n;
+  return 0;
+}
+
+namespace {
+
+template <int N>
+int64_t det_blocks(int64_t nsel) {
+  const int64_t tiles = (nsel + TimeCfg<N>::C - 1) / TimeCfg<N>::C;
+  return (tiles + TIME_DET_TILES - 1) / TIME_DET_TILES;
+}
+
+template <int N, int OUT, bool BLUE>
+cudaError_t launch_n(const TimeArgs& a, cudaStream_t st) {
+  using TC = TimeCfg<N>;
+  const int64_t gx = OUT == TIME_DETECTOR ? det_blocks<N>(a.nsel) : (a.nsel + TC::C - 1) / TC::C;
+  const int64_t gy = std::min<int64_t>(a.P, 65535), gz = (a.P + gy - 1) / gy;
+  if (gx > 0x7fffffff || gz > 65535) return cudaErrorInvalidValue;
+  auto* k = k_time_fft<N, OUT, BLUE>;
+  if (TC::SMEM > 46 * 1024) {
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TC::SMEM);
+    if (e != cudaSuccess) return e;
+  }
+  k<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), TC::THREADS, TC::SMEM, st>>>(a);
+  return cudaGetLastError();
+}
+
+template <int N>
+cudaError_t launch_len(const TimeArgs& a, int out, bool chirp, cudaStream_t st) {
+  if constexpr (fft_pow2(N)) {
+    if (chirp) {
+      if (out == TIME_S) return launch_n<N, TIME_S, true>(a, st);
+      if (out == TIME_DETECTOR) return launch_n<N, TIME_DETECTOR, true>(a, st);
+      return launch_n<N, TIME_TILDE, true>(a, st);
+    }
+  }
+  if constexpr (N <= 2048) {
+    if (out == TIME_S) return launch_n<N, TIME_S, false>(a, st);
+    if (out == TIME_DETECTOR) return launch_n<N, TIME_DETECTOR, false>(a, st);
+    return launch_n<N, TIME_TILDE, false>(a, st);
+  }
+  return cudaErrorInvalidValue;
+}
+
+#define TACAW_TIME_DISPATCH(n, CALL) \
+  switch (n) {                       \
+    case 32: return CALL(32);        \
+    case 64: return CALL(64);        \
+    case 96: return CALL(96);        \
+    case 128: return CALL(128);      \
+    case 192: return CALL(192);      \
+    case 256: return CALL(256);      \
+    case 384: return CALL(384);      \
+    case 512: return CALL(512);      \
+    case 768: return CALL(768);      \
+    case 1024: return CALL(1024);    \
+    case 1152: return CALL(1152);    \
+    case 2048: return CALL(2048);    \
+    case 4096: return CALL(4096);    \
+  }
+
+cudaError_t launch_time_fft(int n, const TimeArgs& a, int out, bool chirp, cudaStream_t st) {
+#define TACAW_CALL(N) launch_len<N>(a, out, chirp, st)
+  TACAW_TIME_DISPATCH(n, TACAW_CALL)
+#undef TACAW_CALL
+  return cudaErrorInvalidValue;
+}
+
+int64_t time_det_blocks(int n, int64_t nsel) {
+#define TACAW_CALL(N) det_blocks<N>(nsel)
+  TACAW_TIME_DISPATCH(n, TACAW_CALL)
+#undef TACAW_CALL
+  return 0;
+}
+
+}  // namespace
+
+int64_t time_fft_parts(int64_t F, int64_t nsel) {
+  bool chirp;
+  const int n = time_fft_length(F, &chirp);
+  return n ? time_det_blocks(n, nsel) : 0;
+}
+
+// S (full, or the spectrum image with REDUCE_DETECTOR) by FFT; the caller has checked
+// time_fft_length.
+int spectrum_fft(tacaw_ctx* ctx, const float2* psi, int64_t P, int64_t F, const SpecIO& io, int32_t reduce, float* S,
+                 Scratch& sc) {
+  TimeArgs a{};
+  bool chirp;
+  const int n = time_fft_length(F, &chirp);
+  a.psi = psi;
+  a.P = P;
+  a.F = a.nf = F;
+  a.in_nq = io.in_nq;
+  a.in_qsel = io.in_qsel;
+  a.nsel = io.nsel;
+  a.out_nq = io.out_nq;
+  a.out_qsel = io.out_qsel;
+  a.tw = ctx->tw;
+  a.S = S;
+  if (chirp) {
+    const int rc = get_chirp(ctx, F, n, &a.chirp, &a.bhat);
+    if (rc != TACAW_OK) return rc;
+  }
+  const bool det = reduce == TACAW_REDUCE_DETECTOR;
+  const int64_t nparts = det ? time_det_blocks(n, io.nsel) : 0;
+  cudaError_t e;
+  if (det && (e = sc.get(&a.part, (size_t)P * nparts * F)) != cudaSuccess) return cuda_err(ctx, e, "detector partial sums");
+  const double pfq = (double)P * F * io.nsel;
+  {
+    ProfScope ps(ctx, "time_fft", sc.st, pfq * 8 + (det ? (double)P * nparts * F * 8 : pfq * 4),
+                 pfq * 5.0 * std::log2((double)std::max<int64_t>(F, 2)));
+    if ((e = launch_time_fft(n, a, det ? TIME_DETECTOR : TIME_S, chirp, sc.st)) != cudaSuccess)
+      return cuda_err(ctx, e, "k_time_fft");
+  }
+  if (det) {
+    ProfScope ps(ctx, "detector_tiles", sc.st, (double)P * nparts * F * 8 + (double)P * F * 4, (double)P * nparts * F);
+    if ((e = launch_detector_parts(a.part, P, F, nparts, S, sc.st)) != cudaSuccess)
+      return cuda_err(ctx, e, "k_detector_parts");
+  }
+  return TACAW_OK;
+}
+
+// psi~ of the frames [f0, f0 + nf) of F against a static reference (tacaw_spectrum_partial).
+int partial_fft(tacaw_ctx* ctx, const float2* psi, const float2* ref, int64_t P, int64_t nf, int64_t f0, int64_t F,
+                int64_t nq, const int32_t* qsel, int64_t nsel, float2* tilde, cudaStream_t st) {
+  TimeArgs a{};
+  bool chirp;
+  const int n = time_fft_length(F, &chirp);
+  a.psi = psi;
+  a.ref = ref;
+  a.P = P;
+  a.F = F;
+  a.nf = nf;
+  a.f0 = f0;
+  a.in_nq = nq;
+  a.in_qsel = qsel;
+  a.nsel = nsel;
+  a.tilde = tilde;
+  a.tw = ctx->tw;
+  if (chirp) {
+    const int rc = get_chirp(ctx, F, n, &a.chirp, &a.bhat);
+    if (rc != TACAW_OK) return rc;
+  }
+  ProfScope ps(ctx, "time_fft_partial", st, (double)P * nsel * 8 * (nf + F), (double)P * nsel * F * 5.0 * std::log2((double)std::max<int64_t>(F, 2)));
+  const cudaError_t e = launch_time_fft(n, a, TIME_TILDE, chirp, st);
+  return e == cudaSuccess ? TACAW_OK : cuda_err(ctx, e, "k_time_fft");
+}
+
+}  // namespace tacaw

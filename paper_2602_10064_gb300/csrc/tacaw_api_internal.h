@@ -88,6 +88,7 @@ struct tacaw_ctx {
   uint64_t ff_version = 0;
   std::map<std::vector<double>, std::unique_ptr<GeoCache>> geos;
   std::map<int64_t, float2*> time_tw;
+  std::map<int64_t, std::pair<float2*, float2*>> chirps;  // chirp-z tables (chirp, spectrum) per F
   std::map<int64_t, std::pair<void*, void*>> dft_ops;  // tensor-core DFT operands (hi, lo) per F and kind
   int* d_status = nullptr;  // device status word: bits TACAW_STATUS_* (tacaw_internal.cuh)
   int64_t max_chunk_frames = 0;  // option: cap on frames per chunk (0 = automatic)
@@ -171,6 +172,16 @@ int get_time_tw(tacaw_ctx* ctx, int64_t F, float2** out);
 // tensor-core epilogue).
 int spectrum_tc(tacaw_ctx* ctx, const float2* psi_k, int64_t P, int64_t F, const SpecIO& io, int32_t precision,
                 int32_t reduce, float* S, Scratch& sc);
+// FFT time transform (k_time_fft.cu).  time_fft_length: the transform length for F frames (0: none),
+// *chirp: F itself is no engine length and goes through the chirp-z convolution.  time_fft_parts:
+// partial sums per probe of the spectrum image.
+int time_fft_length(int64_t F, bool* chirp);
+int64_t time_fft_parts(int64_t F, int64_t nsel);
+int get_chirp(tacaw_ctx* ctx, int64_t F, int M, const float2** chirp, const float2** bhat);
+int spectrum_fft(tacaw_ctx* ctx, const float2* psi, int64_t P, int64_t F, const SpecIO& io, int32_t reduce, float* S,
+                 Scratch& sc);
+int partial_fft(tacaw_ctx* ctx, const float2* psi, const float2* ref, int64_t P, int64_t nf, int64_t f0, int64_t F,
+                int64_t nq, const int32_t* qsel, int64_t nsel, float2* tilde, cudaStream_t st);
 // The whole time transform (mean, residual, DFT, |.|^2, optional detector sum) on P probes.
 int spectrum_impl(tacaw_ctx* ctx, const float2* psi_k, int64_t P, int64_t F, const SpecIO& io, int32_t precision,
                   int32_t reduce, float* S_out, Scratch& sc);

@@ -32,7 +32,7 @@ struct FftPass {
 };
 constexpr FftPass kFftPasses[] = {
     {4, 8},   {8, 8},    {4, 32},   {8, 32},  {16, 32}, {32, 32}, {4, 64},  {8, 64}, {4, 256}, {8, 16},  {16, 16},
-    {16, 64}, {2, 256},  {8, 256},  {4, 12},  {2, 48},  {4, 48},  {2, 192}, {4, 24}, {8, 96},  {6, 24},  {8, 144}};
+    {16, 64}, {16, 256}, {2, 256},  {8, 256},  {4, 12},  {2, 48},  {4, 48},  {2, 192}, {4, 24}, {8, 96},  {6, 24},  {8, 144}};
 // Entries (float2) of the table of a pass.
 constexpr int pass_entries(int r, int ns) { return r == 2 ? ns : 2 * (r / 2) * ns; }
 // Start of its table, in float2 (all sizes are even: the pairs are 16-byte aligned); -1: no such pass.
@@ -221,6 +221,9 @@ cudaError_t launch_residual_f32(const float2* psi, const double2* mean, int64_t 
 // S[p][m][qsel[j]] = |sum_n W[m][n] r[p][n][j]|^2 (FP32), W from the length-F table
 cudaError_t launch_dft_fp32(const float2* r, const float2* twF, int64_t P, int64_t F, int64_t nsel, int64_t nq,
                             const int32_t* qsel, float* S, cudaStream_t st);
+// SI[p][m] = sum over i < nparts of part[p][i][m] (FP64, fixed order)
+cudaError_t launch_detector_parts(const double* part, int64_t P, int64_t F, int64_t nparts, float* SI,
+                                  cudaStream_t st);
 // SI[p][m] = sum_j S[p][m][qsel[j]] (FP64 accumulation, deterministic)
 cudaError_t launch_detector_reduce(const float* S, int64_t P, int64_t F, int64_t nq, const int32_t* qsel,
                                    int64_t nsel, float* SI, cudaStream_t st);
