@@ -27,9 +27,19 @@
 
 namespace tacaw {
 
-__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 operator-(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// Complex sums as packed pairs (one instruction for both parts, each rounded as its scalar form;
+// a - b as a + (-1) b, whose product is exact).
+__device__ __forceinline__ float2 operator+(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 operator-(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 operator*(float s, float2 a) { return make_float2(s * a.x, s * a.y); }
+// s a + b.
+__device__ __forceinline__ float2 fma2(float s, float2 a, float2 b) { return __ffma2_rn(make_float2(s, s), a, b); }
+// a + SIGN i b and a - SIGN i b: the swapped parts need scalar sums (a packed operand would have to
+// be moved into place first).
+template <int SIGN>
+__device__ __forceinline__ float2 add_si(float2 a, float2 b) {
+  return SIGN < 0 ? make_float2(a.x + b.y, a.y - b.x) : make_float2(a.x - b.y, a.y + b.x);
+}
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
   return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
@@ -77,11 +87,11 @@ __device__ __forceinline__ void dft2(float2* u) {
 // X[k] = sum_n u[n] exp(SIGN 2 pi i n k / 4), natural order.
 template <int SIGN>
 __device__ __forceinline__ void dft4(float2& a0, float2& a1, float2& a2, float2& a3) {
-  float2 s02 = a0 + a2, d02 = a0 - a2, s13 = a1 + a3, d13 = mul_si<SIGN>(a1 - a3);
+  float2 s02 = a0 + a2, d02 = a0 - a2, s13 = a1 + a3, d13 = a1 - a3;
   a0 = s02 + s13;
   a2 = s02 - s13;
-  a1 = d02 + d13;
-  a3 = d02 - d13;
+  a1 = add_si<SIGN>(d02, d13);
+  a3 = add_si<-SIGN>(d02, d13);
 }
 
 template <int SIGN>
@@ -99,14 +109,13 @@ __device__ __forceinline__ void dft8(float2* u) {
   const float r2 = 0.70710678118654752f;
   // w8^k = exp(SIGN 2 pi i k / 8)
   float2 t1 = cmul(o1, make_float2(r2, SIGN * r2));
-  float2 t2 = mul_si<SIGN>(o2);
   float2 t3 = cmul(o3, make_float2(-r2, SIGN * r2));
   u[0] = e0 + o0;
   u[4] = e0 - o0;
   u[1] = e1 + t1;
   u[5] = e1 - t1;
-  u[2] = e2 + t2;
-  u[6] = e2 - t2;
+  u[2] = add_si<SIGN>(e2, o2);
+  u[6] = add_si<-SIGN>(e2, o2);
   u[3] = e3 + t3;
   u[7] = e3 - t3;
 }
@@ -142,10 +151,10 @@ template <int SIGN>
 __device__ __forceinline__ void dft3(float2& a0, float2& a1, float2& a2) {
   const float h = 0.86602540378443865f;  // sin(pi / 3)
   const float2 s = a1 + a2, d = mul_si<SIGN>(a1 - a2);
-  const float2 m = a0 - 0.5f * s;
+  const float2 m = fma2(-0.5f, s, a0);
   a0 = a0 + s;
-  a1 = m + h * d;
-  a2 = m - h * d;
+  a1 = fma2(h, d, m);
+  a2 = fma2(-h, d, m);
 }
 
 // exp(SIGN 2 pi i j / 24) (j compile-time after unrolling): the twiddles inside the radix-6,

@@ -131,14 +131,19 @@ static dim3 batch_grid(int gx, int64_t nb) {
   return dim3((unsigned)gx, y, z);
 }
 
+// The compact row accessors with the band read at run time.  Elements e < E / 2 cover x < N / 2,
+// where only x <= mb is in band (c = x), the others x >= N / 2, where only x >= N - mb is
+// (c = x - N + W; with every column kept, mb = N / 2 and W = N, c = x): one comparison of t with a
+// value common to all threads, and a fixed offset from one of two pointers.
 template <int N, int E>
 __device__ __forceinline__ void load_row_compact(float2 (&v)[E], const float2* __restrict__ src, const Band& b,
                                                  int t) {
   constexpr int T = N / E;
+  const float2 *lo = src + t, *hi = src + t + (b.W - N);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int c = band_x_col(b, N, t + T * e);
-    v[e] = c >= 0 ? src[c] : make_float2(0.f, 0.f);
+    const bool in = e < E / 2 ? t <= b.mb - T * e : t >= N - b.mb - T * e;
+    v[e] = in ? (e < E / 2 ? lo : hi)[T * e] : make_float2(0.f, 0.f);
   }
 }
 
@@ -146,10 +151,11 @@ template <int N, int E>
 __device__ __forceinline__ void store_row_compact(const float2 (&v)[E], float2* __restrict__ dst, const Band& b,
                                                   int t) {
   constexpr int T = N / E;
+  float2 *lo = dst + t, *hi = dst + t + (b.W - N);
 #pragma unroll
   for (int e = 0; e < E; ++e) {
-    const int c = band_x_col(b, N, t + T * e);
-    if (c >= 0) dst[c] = v[e];
+    const bool in = e < E / 2 ? t <= b.mb - T * e : t >= N - b.mb - T * e;
+    if (in) (e < E / 2 ? lo : hi)[T * e] = v[e];
   }
 }
 
