@@ -12,6 +12,8 @@
 // Between the passes only the in-band columns (|kx| <= kbl) are kept, in compact order.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "fft.cuh"
 #include "tacaw_internal.cuh"
 
@@ -797,21 +799,26 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Most probes of a frame that one CTA of the slice row pass takes through its rows.  One probe a CTA
+// copied the transmission row (60% of the pass's reads) once for every probe and waited for every
+// wave's row; with eight, 256 points x 2048 waves take 300 us instead of 360.
+constexpr int SLICE_ROW_PROBES = 8;
+
 // MB >= 0: the band's half-width, fixed at compile time (the standard 2/3 band of a square
 // cell, MB = NX / 3); MB < 0: read from b.
 template <int NX, bool FIRST, bool PLANE, bool TF, int MB = -1>
 __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW, NX, SliceRowCfg<NX>>())
     k_slice_row(Geo geo, Band b, const float2* __restrict__ Apsi, const float2* __restrict__ psi0,
-                const float2* __restrict__ ttab, int S, int s, int nfc, int nwaves, float plane_amp,
+                const float2* __restrict__ ttab, int S, int s, int P, int ppb, int nfc, int nbatch, float plane_amp,
                 float2* __restrict__ Bpsi) {
   constexpr int E = SliceRowCfg<NX>::E, T = SliceRowCfg<NX>::T, G = SliceRowCfg<NX>::G;
   constexpr int PL = Tuned<K_SLICE_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
-  const int w = batch_index();
-  if (w >= nwaves) return;
+  const int bi = batch_index();
+  if (bi >= nbatch) return;
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
-  const int p = w / nfc, fl = w - p * nfc;
+  const int pg = bi / nfc, fl = bi - pg * nfc, p0 = pg * ppb, p1 = p0 + ppb < P ? p0 + ppb : P;
   const RowIdx<NX, E> idx{g * row_smem_stride<NX, E>()};
   const auto sync = group_sync<T>(g);
   float2 v[E];
@@ -820,7 +827,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
     load_row_compact<NX>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = (plane_amp * (float)NX) * v[e];
-    store_row_compact<NX>(v, Bpsi + ((size_t)w * ny + y) * b.Wp, b, t);
+    store_row_compact<NX>(v, Bpsi + ((size_t)bi * ny + y) * b.Wp, b, t);
     return;
   }
   // The transmission row goes to a shared-memory stash before it is used; each thread writes
@@ -839,25 +846,37 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
     for (int e = 0; e < E; ++e) cp_async8(tst + t + T * e, trow + t + T * e);
     asm volatile("cp.async.commit_group;" ::: "memory");
   }
-  if (FIRST) {
-    if (!TF) cp_async_wait_all();
-    if (PLANE) {
+  // The probes p0 .. p1 - 1 of this frame share the stashed row: the row of the next probe's wave is
+  // loaded while this one's is transformed.
+  const auto load = [&](float2 (&u)[E], int p) {
+    if (!FIRST) {
+      load_row<NX, MB>(u, Apsi + ((size_t)(p * nfc + fl) * ny + y) * b.Wp, b, t);
+    } else if (PLANE) {
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = plane_amp * tst[t + T * e];
+      for (int e = 0; e < E; ++e) u[e] = make_float2(plane_amp, 0.f);
     } else {
       const float2* src = psi0 + ((size_t)p * ny + y) * NX;
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = cmul(src[t + T * e], tst[t + T * e]);
+      for (int e = 0; e < E; ++e) u[e] = src[t + T * e];
     }
-  } else {
-    load_row<NX, MB>(v, Apsi + ((size_t)w * ny + y) * b.Wp, b, t);
-    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
+  };
+  load(v, p0);
+  for (int p = p0; p < p1; ++p) {
+    float2 next[E];
+    if (!TF && p + 1 < p1) load(next, p + 1);
+    if (!FIRST) fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
     if (!TF) cp_async_wait_all();
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = cmul(v[e], tst[t + T * e]);
+    for (int e = 0; e < E; ++e) {
+      if (FIRST && PLANE) v[e] = plane_amp * tst[t + T * e];
+      else v[e] = cmul(v[e], tst[t + T * e]);
+    }
+    fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
+    store_row<NX, MB>(v, Bpsi + ((size_t)(p * nfc + fl) * ny + y) * b.Wp, b, t);
+    if (TF) return;  // one probe
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = next[e];
   }
-  fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
-  store_row<NX, MB>(v, Bpsi + ((size_t)w * ny + y) * b.Wp, b, t);
 }
 
 // WPC > 0: the row stride of the compact columns (Wp) fixed at compile time (the standard band
@@ -1162,15 +1181,20 @@ template <int NX>
 static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane, int tfused, const float2* Apsi,
                                const float2* psi0, const float2* t, int S, int s, int P, int nfc, float plane_amp,
                                float2* Bpsi, int static_band, cudaStream_t st) {
-  const int nw = P * nfc;
-  const dim3 grid = batch_grid(g.ny / SliceRowCfg<NX>::G, nw);
+  // probes per CTA: up to SLICE_ROW_PROBES, while at least 16 CTAs are left for every SM
   constexpr int TH = SliceRowCfg<NX>::THREADS;
+  const int64_t ctas = (int64_t)P * nfc * (g.ny / SliceRowCfg<NX>::G);
+  int ppb = (int)std::min<int64_t>(std::min(P, SLICE_ROW_PROBES), std::max<int64_t>(1, ctas / (16 * 152)));
+  ppb = (P + (P + ppb - 1) / ppb - 1) / ((P + ppb - 1) / ppb);  // even groups
+  const int nbatch = (P + ppb - 1) / ppb * nfc;
+  const dim3 grid = batch_grid(g.ny / SliceRowCfg<NX>::G, nbatch);
 #define TACAW_SLICE_ROW(F, PL, TFU)                                                                               \
   do {                                                                                                            \
     constexpr int SM = SliceRowSmem<NX, TFU>::BYTES;                                                              \
     cudaError_t e_ = prep(k_slice_row<NX, F, PL, TFU>, SM);                                                       \
     if (e_ != cudaSuccess) return e_;                                                                             \
-    k_slice_row<NX, F, PL, TFU><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, nfc, nw, plane_amp, Bpsi);        \
+    k_slice_row<NX, F, PL, TFU><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch, plane_amp,      \
+                                                       Bpsi);                                                     \
   } while (0)
   // the later slices (all but one of S) with the standard band fixed at compile time
   constexpr int MB3 = NX / 3;
@@ -1181,8 +1205,8 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
     constexpr int SM = SliceRowSmem<NX, TFU>::BYTES;                                                              \
     cudaError_t e_ = prep(k_slice_row<NX, false, false, TFU, MB3>, SM);                                           \
     if (e_ != cudaSuccess) return e_;                                                                             \
-    k_slice_row<NX, false, false, TFU, MB3><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, nfc, nw, plane_amp,  \
-                                                                  Bpsi);                                          \
+    k_slice_row<NX, false, false, TFU, MB3><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch,  \
+                                                                  plane_amp, Bpsi);                               \
   } while (0)
   if (tfused) {
     if (first && plane) TACAW_SLICE_ROW(true, true, true);
