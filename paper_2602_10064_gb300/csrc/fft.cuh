@@ -283,11 +283,12 @@ __device__ __forceinline__ void dft_r(float2* u) {
 __host__ __device__ constexpr bool fft_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
 // Elements per thread (E) for a transform of length N: 8 or 16 for powers of two (8 for
-// N <= 64), 24 for 768 and 1152 (three passes), 12 for the other lengths with a factor 3.  A
-// kernel picks E per pass direction (powers of two); T = N / E threads share one transform.
+// N <= 64), 24 for the lengths with a factor 3: two passes for 96 and 192, three for the others
+// (8 x 8 x 12 beats 24 x 4 x 8 for 768 by 10%, but 8 x 12 x 12 loses to 24 x 6 x 8 for 1152 by 10%).  A kernel picks E per pass direction (powers of two); T = N / E threads share one
+// transform.
 template <int N, int EPREF>
 struct FftPlan {
-  static constexpr int E = fft_pow2(N) ? ((N <= 64) ? 8 : EPREF) : ((N == 768 || N == 1152) ? 24 : 12);
+  static constexpr int E = fft_pow2(N) ? ((N <= 64) ? 8 : EPREF) : 24;
   static constexpr int T = N / E;
 };
 
@@ -310,14 +311,13 @@ struct GroupSync {
   }
 };
 
-// Shared-memory padding: one slot per 2^SH elements along the transform, 2^SH = E for 8, 16
-// and 32 elements per thread (16 for 12 and 24).  The first pass of every plan stores each
-// thread's E outputs contiguously (stride E across the threads of a warp); with one pad per E
-// those 64-bit stores, and the own-position reads of every pass, stay at (or near) the minimum
-// two wavefronts per warp.
+// Shared-memory padding: one slot per 2^SH elements along the transform.  The first pass of every
+// plan stores each thread's R1 outputs contiguously (stride R1 across the threads of a warp); the pad
+// makes that stride odd, so that those 64-bit stores, and the own-position reads of every pass, stay
+// at (or near) the minimum two wavefronts per warp.
 template <int N, int E>
 struct PadShift {
-  static constexpr int SH = (E == 8 || N <= 64) ? 3 : (E == 32 ? 5 : 4);
+  static constexpr int SH = E == 24 ? (N == 96 ? 2 : N == 1152 ? 4 : 3) : (E == 8 || N <= 64) ? 3 : (E == 32 ? 5 : 4);
 };
 template <int N, int E>
 struct RowIdx {
@@ -465,23 +465,20 @@ __device__ __forceinline__ void fft(float2 (&v)[E], float2* sm, const Idx& idx, 
     fft_pass<4096, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<4096, E, 16, 16, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<4096, E, 16, 256, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 12 && N == 96) {
+  } else if constexpr (E == 24 && N == 96) {
     fft_pass<96, E, 12, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<96, E, 4, 12, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<96, E, 2, 48, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 12 && N == 192) {
-    fft_pass<192, E, 12, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<192, E, 4, 12, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<192, E, 4, 48, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 12 && N == 384) {
-    fft_pass<384, E, 12, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<384, E, 4, 12, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<384, E, 4, 48, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<384, E, 2, 192, SIGN, true>(v, sm, idx, t, tw, sync);
+    fft_pass<96, E, 8, 12, SIGN, true>(v, sm, idx, t, tw, sync);
+  } else if constexpr (E == 24 && N == 192) {
+    fft_pass<192, E, 24, 1, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<192, E, 8, 24, SIGN, true>(v, sm, idx, t, tw, sync);
+  } else if constexpr (E == 24 && N == 384) {
+    fft_pass<384, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<384, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<384, E, 6, 64, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (E == 24 && N == 768) {
-    fft_pass<768, E, 24, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<768, E, 4, 24, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<768, E, 8, 96, SIGN, true>(v, sm, idx, t, tw, sync);
+    fft_pass<768, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<768, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
+    fft_pass<768, E, 12, 64, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (E == 24 && N == 1152) {
     fft_pass<1152, E, 24, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<1152, E, 6, 24, SIGN, false>(v, sm, idx, t, tw, sync);

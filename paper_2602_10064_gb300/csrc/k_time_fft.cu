@@ -33,7 +33,7 @@ namespace tacaw {
 // 16 or 32 whole lines; more columns of the long transforms would leave one CTA per SM.
 template <int N>
 struct TimeCfg {
-  static constexpr int E = N <= 64 ? 8 : (N == 768 || N == 1152) ? 24 : fft_pow2(N) ? (N >= 2048 ? 32 : 16) : 12;
+  static constexpr int E = !fft_pow2(N) ? 24 : N <= 64 ? 8 : N >= 2048 ? 32 : 16;
   static constexpr int T = N / E;
   static constexpr int C = N <= 128 ? 32 : N <= 512 ? 16 : N <= 2048 ? 8 : 4;
   static constexpr int THREADS = T * C;

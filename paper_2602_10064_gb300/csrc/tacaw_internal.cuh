@@ -32,7 +32,7 @@ struct FftPass {
 };
 constexpr FftPass kFftPasses[] = {
     {4, 8},   {8, 8},    {4, 32},   {8, 32},  {16, 32}, {32, 32}, {4, 64},  {8, 64}, {4, 256}, {8, 16},  {16, 16},
-    {16, 64}, {16, 256}, {2, 256},  {8, 256},  {4, 12},  {2, 48},  {4, 48},  {2, 192}, {4, 24}, {8, 96},  {6, 24},  {8, 144}};
+    {16, 64}, {16, 256}, {2, 256}, {8, 256}, {8, 12}, {8, 24}, {6, 64}, {12, 64}, {6, 24}, {8, 144}};
 // Entries (float2) of the table of a pass.
 constexpr int pass_entries(int r, int ns) { return r == 2 ? ns : 2 * (r / 2) * ns; }
 // Start of its table, in float2 (all sizes are even: the pairs are 16-byte aligned); -1: no such pass.
