@@ -29,7 +29,7 @@ namespace tacaw {
 // tuner's measurement builds).
 enum KernelId {
   K_SPLAT_ROW, K_COL_POT, K_ROW_POT_OUT, K_ROW_VT, K_COL_T, K_ROW_TOUT, K_PROBE_COL, K_PROBE_ROW,
-  K_SLICE_ROW, K_SLICE_COL
+  K_SLICE_ROW, K_SLICE_COL, K_SLICE_ROW_SCAN
 };
 }  // namespace tacaw
 #include "tuning_table.h"
@@ -101,7 +101,9 @@ template <int N> using PotOutCfg = RowCfg<N, Tuned<K_ROW_POT_OUT, N>::EV>;
 template <int N> using RowVtCfg = RowCfg<N, Tuned<K_ROW_VT, N>::EV>;
 template <int N> using RowToutCfg = RowCfg<N, Tuned<K_ROW_TOUT, N>::EV>;
 template <int N> using ProbeRowCfg = RowCfg<N, Tuned<K_PROBE_ROW, N>::EV>;
-template <int N> using SliceRowCfg = RowCfg<N, Tuned<K_SLICE_ROW, N>::EV>;
+// one probe (the compact t, TF) and several (the full t) have different loops: tuned apart
+template <bool TF> __host__ __device__ constexpr int slice_row_id() { return TF ? K_SLICE_ROW : K_SLICE_ROW_SCAN; }
+template <int N, bool TF> using SliceRowCfg = RowCfg<N, Tuned<slice_row_id<TF>(), N>::EV>;
 template <int N> using ColPotCfg = ColCfg<N, Tuned<K_COL_POT, N>::WIDE, Tuned<K_COL_POT, N>::EV>;
 template <int N> using ColTCfg = ColCfg<N, Tuned<K_COL_T, N>::WIDE, Tuned<K_COL_T, N>::EV>;
 template <int N> using ProbeColCfg = ColCfg<N, Tuned<K_PROBE_COL, N>::WIDE, Tuned<K_PROBE_COL, N>::EV>;
@@ -789,7 +791,7 @@ __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW,
 // Shared memory of the slice row pass: the FFT scratch, plus (TF) one stashed t row per group.
 template <int NX, bool TF>
 struct SliceRowSmem {
-  static constexpr int BYTES = SliceRowCfg<NX>::SMEM + SliceRowCfg<NX>::G * NX * (int)sizeof(float2);
+  static constexpr int BYTES = SliceRowCfg<NX, TF>::SMEM + SliceRowCfg<NX, TF>::G * NX * (int)sizeof(float2);
 };
 
 // Asynchronous 8-byte copy global -> shared (completes at cp_async_wait_all of the same thread).
@@ -799,6 +801,9 @@ __device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) 
 }
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
+// Most waves that one CTA of the slice column pass takes through its columns.  256 points, 2304 waves,
+// 16 elements a thread: 2.97 ms for 8 slices with the loop; 4.16 with 32 elements, which spill in it.
+constexpr int SLICE_COL_WAVES = 8;
 // Most probes of a frame that one CTA of the slice row pass takes through its rows.  One probe a CTA
 // copied the transmission row (60% of the pass's reads) once for every probe and waited for every
 // wave's row; with eight, 256 points x 2048 waves take 300 us instead of 360.
@@ -807,12 +812,13 @@ constexpr int SLICE_ROW_PROBES = 8;
 // MB >= 0: the band's half-width, fixed at compile time (the standard 2/3 band of a square
 // cell, MB = NX / 3); MB < 0: read from b.
 template <int NX, bool FIRST, bool PLANE, bool TF, int MB = -1>
-__global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW, NX, SliceRowCfg<NX>>())
+__global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_row_id<TF>(), NX, SliceRowCfg<NX, TF>>())
     k_slice_row(Geo geo, Band b, const float2* __restrict__ Apsi, const float2* __restrict__ psi0,
                 const float2* __restrict__ ttab, int S, int s, int P, int ppb, int nfc, int nbatch, float plane_amp,
                 float2* __restrict__ Bpsi) {
-  constexpr int E = SliceRowCfg<NX>::E, T = SliceRowCfg<NX>::T, G = SliceRowCfg<NX>::G;
-  constexpr int PL = Tuned<K_SLICE_ROW, NX>::PLAN;
+  using RC = SliceRowCfg<NX, TF>;
+  constexpr int E = RC::E, T = RC::T, G = RC::G;
+  constexpr int PL = Tuned<slice_row_id<TF>(), NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int bi = batch_index();
@@ -834,18 +840,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
   // and rereads only its own positions, so no barrier is needed.  TF: t is inverse-transformed
   // first (only one row of the wave is then live in registers).  Otherwise the full t row is
   // copied asynchronously at once, so its load overlaps the wave's load and inverse transform.
-  float2* tst = reinterpret_cast<float2*>(smraw + SliceRowCfg<NX>::SMEM) + g * NX;
-  if (TF) {
-    load_row<NX, MB>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
-    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
-#pragma unroll
-    for (int e = 0; e < E; ++e) tst[t + T * e] = v[e];
-  } else {
-    const float2* trow = ttab + ((size_t)(fl * S + s) * ny + y) * NX;
-#pragma unroll
-    for (int e = 0; e < E; ++e) cp_async8(tst + t + T * e, trow + t + T * e);
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  }
+  float2* tst = reinterpret_cast<float2*>(smraw + RC::SMEM) + g * NX;
   // The probes p0 .. p1 - 1 of this frame share the stashed row: the row of the next probe's wave is
   // loaded while this one's is transformed.
   const auto load = [&](float2 (&u)[E], int p) {
@@ -860,9 +855,23 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
       for (int e = 0; e < E; ++e) u[e] = src[t + T * e];
     }
   };
-  load(v, p0);
+  float2 next[E];
+  if (TF) {
+    load_row<NX, MB>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
+    load(next, p0);
+    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
+#pragma unroll
+    for (int e = 0; e < E; ++e) tst[t + T * e] = v[e];
+#pragma unroll
+    for (int e = 0; e < E; ++e) v[e] = next[e];
+  } else {
+    const float2* trow = ttab + ((size_t)(fl * S + s) * ny + y) * NX;
+#pragma unroll
+    for (int e = 0; e < E; ++e) cp_async8(tst + t + T * e, trow + t + T * e);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    load(v, p0);
+  }
   for (int p = p0; p < p1; ++p) {
-    float2 next[E];
     if (!TF && p + 1 < p1) load(next, p + 1);
     if (!FIRST) fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
     if (!TF) cp_async_wait_all();
@@ -881,37 +890,67 @@ __global__ void __launch_bounds__(SliceRowCfg<NX>::THREADS, minb_of<K_SLICE_ROW,
 
 // WPC > 0: the row stride of the compact columns (Wp) fixed at compile time (the standard band
 // of a square grid), so the strided loads and stores take immediate offsets; else Wp.
-template <int NY, bool LAST, int WPC = -1>
+// LOOP: a CTA takes its columns of wpb waves one after the other.  The propagator times mask and
+// scale is put together once per CTA, in shared memory (each thread reads back only what it wrote),
+// and the next wave's column is loaded while this one is transformed.  Both forms multiply by the
+// same product, so that a wave's bits do not depend on how many waves a launch holds.
+template <int NY>
+__host__ __device__ constexpr bool slice_col_loop() {
+  return 2 * SliceColCfg<NY>::SMEM <= 100 * 1024;  // two such CTAs per SM
+}
+template <int NY, bool LAST, bool LOOP, int WPC = -1>
 __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL, NY, SliceColCfg<NY>>())
     k_slice_col(Geo geo, Band b, const float2* __restrict__ Bpsi, const float2* __restrict__ px,
-                const float2* __restrict__ py, float scale, int nfc, int nwaves, int64_t F_total, int64_t f0,
+                const float2* __restrict__ py, float scale, int wpb, int nfc, int nwaves, int64_t F_total, int64_t f0,
                 const int2* __restrict__ disc, int64_t nsel, float2* __restrict__ Apsi, float2* __restrict__ psi_k) {
   using CC = SliceColCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
   constexpr int PL = Tuned<K_SLICE_COL, NY>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
-  const int w = batch_index();
-  if (w >= nwaves) return;
+  const int w0 = batch_index() * wpb, w1 = w0 + wpb < nwaves ? w0 + wpb : nwaves;
+  if (w0 >= nwaves) return;
   const int Wp = WPC > 0 ? WPC : b.Wp;
   const int c = threadIdx.x % C, t = threadIdx.x / C, cc = blockIdx.x * C + c;
   const ColIdx<C, CC::SH> idx{c};
   const BlockSync sync;
   const float2* tw = geo.tw;
-  const float2* src = Bpsi + (size_t)w * NY * Wp + cc;
-  float2 v[E];
+  const auto load = [&](float2 (&u)[E], int w) {
+    const float2* src = Bpsi + (size_t)w * NY * Wp + cc;
 #pragma unroll
-  for (int e = 0; e < E; ++e) v[e] = src[(size_t)(t + T * e) * Wp];
-  fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+    for (int e = 0; e < E; ++e) u[e] = src[(size_t)(t + T * e) * Wp];
+  };
+  float2 v[E];
+  load(v, w0);
   const int nb = cc < b.W ? b.colnb[cc] : -1;
   const float2 pxc = cc < b.W ? px[cc] : make_float2(0.f, 0.f);
+  float2* prop = reinterpret_cast<float2*>(smraw + CC::SMEM) + threadIdx.x;  // [E][THREADS]
+  if (LOOP) {
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    const int row = t + T * e, n = fftfreq_index(row, NY);
-    v[e] = (abs(n) <= nb) ? scale * cmul(cmul(v[e], pxc), py[row]) : make_float2(0.f, 0.f);
+    for (int e = 0; e < E; ++e) {
+      const int row = t + T * e, n = fftfreq_index(row, NY);
+      prop[CC::THREADS * e] = (abs(n) <= nb) ? scale * cmul(pxc, py[row]) : make_float2(0.f, 0.f);
+    }
   }
-  if (LAST) {
-    if (cc < b.W) {
+  for (int w = w0; w < w1; ++w) {
+    float2 next[E];
+    if (LOOP && w + 1 < w1) load(next, w + 1);
+    fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      if (LOOP) {
+        v[e] = cmul(v[e], prop[CC::THREADS * e]);
+      } else {
+        const int row = t + T * e, n = fftfreq_index(row, NY);
+        v[e] = cmul(v[e], (abs(n) <= nb) ? scale * cmul(pxc, py[row]) : make_float2(0.f, 0.f));
+      }
+    }
+    if (!LAST) {
+      fft<NY, +1, PL>(v, sm, idx, t, tw, sync);
+      float2* dst = Apsi + (size_t)w * NY * Wp + cc;
+#pragma unroll
+      for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = v[e];
+    } else if (cc < b.W) {
       const int p = w / nfc, fl = w - p * nfc;
       if (disc) {
         // compact exit wave: the in-band points of the disc only, in ascending q = y nx + x;
@@ -934,12 +973,10 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
         for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * geo.nx] = v[e];
       }
     }
-    return;
-  }
-  fft<NY, +1, PL>(v, sm, idx, t, tw, sync);
-  float2* dst = Apsi + (size_t)w * NY * Wp + cc;
+    if (!LOOP) return;  // one wave
 #pragma unroll
-  for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = v[e];
+    for (int e = 0; e < E; ++e) v[e] = next[e];
+  }
 }
 
 // ============================================================================================
@@ -1182,15 +1219,15 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
                                const float2* psi0, const float2* t, int S, int s, int P, int nfc, float plane_amp,
                                float2* Bpsi, int static_band, cudaStream_t st) {
   // probes per CTA: up to SLICE_ROW_PROBES, while at least 16 CTAs are left for every SM
-  constexpr int TH = SliceRowCfg<NX>::THREADS;
-  const int64_t ctas = (int64_t)P * nfc * (g.ny / SliceRowCfg<NX>::G);
+  const int G = tfused ? SliceRowCfg<NX, true>::G : SliceRowCfg<NX, false>::G;
+  const int64_t ctas = (int64_t)P * nfc * (g.ny / G);
   int ppb = (int)std::min<int64_t>(std::min(P, SLICE_ROW_PROBES), std::max<int64_t>(1, ctas / (16 * 152)));
   ppb = (P + (P + ppb - 1) / ppb - 1) / ((P + ppb - 1) / ppb);  // even groups
   const int nbatch = (P + ppb - 1) / ppb * nfc;
-  const dim3 grid = batch_grid(g.ny / SliceRowCfg<NX>::G, nbatch);
+  const dim3 grid = batch_grid(g.ny / G, nbatch);
 #define TACAW_SLICE_ROW(F, PL, TFU)                                                                               \
   do {                                                                                                            \
-    constexpr int SM = SliceRowSmem<NX, TFU>::BYTES;                                                              \
+    constexpr int SM = SliceRowSmem<NX, TFU>::BYTES, TH = SliceRowCfg<NX, TFU>::THREADS;                          \
     cudaError_t e_ = prep(k_slice_row<NX, F, PL, TFU>, SM);                                                       \
     if (e_ != cudaSuccess) return e_;                                                                             \
     k_slice_row<NX, F, PL, TFU><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch, plane_amp,      \
@@ -1202,7 +1239,7 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
   const bool std_band = tacaw::std_band<NX>(b, static_band);
 #define TACAW_SLICE_ROW_STD(TFU)                                                                                   \
   do {                                                                                                            \
-    constexpr int SM = SliceRowSmem<NX, TFU>::BYTES;                                                              \
+    constexpr int SM = SliceRowSmem<NX, TFU>::BYTES, TH = SliceRowCfg<NX, TFU>::THREADS;                          \
     cudaError_t e_ = prep(k_slice_row<NX, false, false, TFU, MB3>, SM);                                           \
     if (e_ != cudaSuccess) return e_;                                                                             \
     k_slice_row<NX, false, false, TFU, MB3><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch,  \
@@ -1241,28 +1278,36 @@ static cudaError_t slice_col_n(const Geo& g, const Band& b, int last, const floa
                                cudaStream_t st) {
   const int nw = P * nfc;
   using CC = SliceColCfg<NY>;
-  const dim3 grid = batch_grid(col_blocks(b, CC::C), nw);
-  constexpr int TH = CC::THREADS, SM = CC::SMEM;
+  constexpr int TH = CC::THREADS;
+  const int cb = col_blocks(b, CC::C);
+  // waves per CTA: up to SLICE_COL_WAVES, while at least 16 CTAs are left for every SM
+  int wpb = 1;
+  if (slice_col_loop<NY>() && !last)
+    wpb = (int)std::min<int64_t>(SLICE_COL_WAVES, std::max<int64_t>(1, (int64_t)nw * cb / (16 * 152)));
+  const dim3 grid = batch_grid(cb, (nw + wpb - 1) / wpb);
+#define TACAW_SLICE_COL(L, LOOP, ...)                                                                                 \
+  do {                                                                                                                \
+    constexpr int SM = CC::SMEM + ((LOOP) ? NY * CC::C * (int)sizeof(float2) : 0);                                      \
+    cudaError_t e_ = prep(k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>, SM);                                   \
+    if (e_ != cudaSuccess) return e_;                                                                                 \
+    k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>                                                               \
+        <<<grid, TH, SM, st>>>(g, b, Bpsi, px, py, scale, wpb, nfc, nw, F_total, f0, disc, nsel, Apsi, psi_k);        \
+    return cudaGetLastError();                                                                                        \
+  } while (0)
+  if (last) TACAW_SLICE_COL(true, false);
   // the later slices of a square grid with the standard band: row stride fixed at compile time
   if constexpr (std_band_built<NY>()) {
     constexpr int WP = std_band_wp(NY);
-    if (!last && g.nx == NY && b.Wp == WP && std_band<NY>(b, static_band)) {
-      cudaError_t e = prep(k_slice_col<NY, false, WP>, SM);
-      if (e != cudaSuccess) return e;
-      k_slice_col<NY, false, WP><<<grid, TH, SM, st>>>(g, b, Bpsi, px, py, scale, nfc, nw, F_total, f0, disc, nsel,
-                                                       Apsi, psi_k);
-      return cudaGetLastError();
+    if (g.nx == NY && b.Wp == WP && std_band<NY>(b, static_band)) {
+      if constexpr (slice_col_loop<NY>())
+        if (wpb > 1) TACAW_SLICE_COL(false, true, WP);
+      TACAW_SLICE_COL(false, false, WP);
     }
   }
-  cudaError_t e = last ? prep(k_slice_col<NY, true>, SM) : prep(k_slice_col<NY, false>, SM);
-  if (e != cudaSuccess) return e;
-  if (last)
-    k_slice_col<NY, true><<<grid, TH, SM, st>>>(g, b, Bpsi, px, py, scale, nfc, nw, F_total, f0, disc, nsel, Apsi,
-                                                psi_k);
-  else
-    k_slice_col<NY, false><<<grid, TH, SM, st>>>(g, b, Bpsi, px, py, scale, nfc, nw, F_total, f0, disc, nsel, Apsi,
-                                                 psi_k);
-  return cudaGetLastError();
+  if constexpr (slice_col_loop<NY>())
+    if (wpb > 1) TACAW_SLICE_COL(false, true);
+  TACAW_SLICE_COL(false, false);
+#undef TACAW_SLICE_COL
 }
 cudaError_t launch_slice_col(const Geo& g, const Band& b, int last, const float2* Bpsi, const float2* px,
                              const float2* py, float scale, int P, int nfc, int64_t F_total, int64_t f0,

@@ -22,40 +22,48 @@ Needs a GPU.  Synthetic inputs come from the repository's `workloads` module.
 from __future__ import annotations
 
 import argparse
+import concurrent.futures as cf
 import json
 import os
+import shutil
 import subprocess
 import sys
+import tempfile
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 
-# kernel class (library profiler name) -> KernelId in k_slices.cu
+# kernel class (library profiler name; the slice row pass of one probe and of several are two) ->
+# KernelId in k_slices.cu
 KERNEL_IDS = {"splat_row": 0, "col_pot": 1, "row_pot_t": 2, "row_vt": 3, "col_t": 4, "row_tout": 5,
-              "slice_row": 8, "slice_col": 9}
+              "slice_row": 8, "slice_col": 9, "slice_row_scan": 10}
 # classes whose kernels take the column-width bit (variant & 4); the others ignore it
 COLUMN_CLASSES = {"col_pot", "col_t", "slice_col"}
-N_KERNELS = 10
+N_KERNELS = 11
 LENGTHS = (32, 64, 128, 256, 512, 1024, 96, 192, 384, 768, 1152)
+TUNED_LENGTHS = LENGTHS[1:]
 MIN_GAIN = 0.02
 
 
 def cases():
-    """(name, transform length, workload factory): runs whose kernel mix matches the hot path
-    at each length (plane waves, and a probe scan for the full-t row pass)."""
+    """(transform length, workload factory): a plane wave and a 6 x 6 probe scan at each length, with
+    the frames for about 1e8 grid points times slices (the launches fill the device several times)."""
     sys.path.insert(0, ROOT)
     import workloads
-    return [
-        ("diamond-128", 128, lambda: workloads.diamond_si(n_frames=512, grid=128, n_slices=8, seed=11)),
-        ("diamond-256", 256, lambda: workloads.diamond_si(n_frames=256, grid=256, n_slices=20, seed=12,
-                                                           reps=(4, 4, 2))),
-        ("scan-256", 256, lambda: workloads.config3(n_frames=16, seed=13)),
-        ("rocksalt-512", 512, lambda: workloads.config2(n_frames=128, seed=14)),
-        ("diamond-1024", 1024, lambda: workloads.config4(n_frames=64, seed=15)),
-        ("diamond-768", 768, lambda: workloads.diamond_si(n_frames=64, grid=768, n_slices=20, seed=16,
-                                                           reps=(8, 8, 2))),
-        ("minimal-example-1152", 1152, lambda: workloads.minimal_example_si(n_frames=16, seed=17)),
-    ]
+    out = []
+    for n in TUNED_LENGTHS:
+        r, S = max(2, n // 50), 8
+        for scan in (0, 6):
+            F = max(8, min(512, int(1.5e8 / (n * n * S)))) if not scan else max(4, min(64, int(4e7 / (n * n * S))))
+
+            def make(n=n, r=r, S=S, scan=scan, F=F):
+                w = workloads.diamond_si(n_frames=F, grid=n, n_slices=S, seed=n + scan, reps=(r, r, 2))
+                if scan:
+                    w.alpha_mrad, w.probes = 30.0, workloads.probe_grid(w.cell[0], w.cell[1], scan)
+                return w
+
+            out.append((n, make))
+    return out
 
 
 def measure(steps: int = 3) -> dict:
@@ -65,17 +73,15 @@ def measure(steps: int = 3) -> dict:
     import paper_2602_10064_gb300 as T
     out = {}
     ctx = T.Context(0)
-    st = torch.cuda.current_stream()
-    for name, n, make in cases():
+    for n, make in cases():
         w = make()
         ctx.load_form_factors(w.form_Z, w.form_coef)
         params, probe = T.params_of(w), T.probe_of(w)
         pos = torch.from_numpy(w.pos).cuda()
         Z = torch.from_numpy(w.Z).cuda()
-        S = torch.empty((w.n_probes, w.n_frames, w.ny, w.nx), dtype=torch.float32, device="cuda")
 
         def run():
-            T.tacaw_run(ctx.h, params, pos, Z, w.n_atoms, w.n_frames, probe, T.DFT_BF16X3, T.REDUCE_NONE, S, st)
+            ctx.run(params, pos, Z, probe, reduce=T.REDUCE_DETECTOR)
 
         def transmission(V):
             ctx.transmission(params, V)
@@ -93,6 +99,8 @@ def measure(steps: int = 3) -> dict:
                 prof = T.tacaw_profile_end(ctx.h)
                 cur = {}
                 for cls, (ms, _n, _b, _f) in prof.items():
+                    if cls == "slice_row" and w.n_probes > 1:
+                        cls = "slice_row_scan"
                     if cls in KERNEL_IDS:
                         cur[cls] = cur.get(cls, 0.0) + ms
                 for cls, ms in cur.items():
@@ -100,10 +108,19 @@ def measure(steps: int = 3) -> dict:
                     best[key] = min(best.get(key, float("inf")), ms)
         for key, ms in best.items():
             out[key] = out.get(key, 0.0) + ms
-        del pos, Z, S, V
+        del pos, Z, V
     ctx.check()
     ctx.close()
     return out
+
+
+def effective(v: int, cls: str, n: int) -> int:
+    """The variant without the bits that change nothing for this kernel and length."""
+    if n not in (512, 1024) or v & 8:
+        v &= ~1
+    if n & (n - 1) or n < 128:
+        v &= ~8
+    return v if cls in COLUMN_CLASSES else v & ~4
 
 
 def choose(results: dict) -> list:
@@ -117,7 +134,7 @@ def choose(results: dict) -> list:
         base = results[0][key]
         v_best, t_best = 0, base
         for v, r in results.items():
-            if (v & 4) and cls not in COLUMN_CLASSES:
+            if v != effective(v, cls, int(n)):
                 continue
             if key in r and r[key] < t_best:
                 v_best, t_best = v, r[key]
@@ -146,10 +163,10 @@ def header(table: list, results: dict) -> str:
               "constexpr int kTunedLengths[11] = {" + ", ".join(str(n) for n in LENGTHS) + "};",
               "",
               "// [kernel][index of N in kTunedLengths]",
-              "constexpr int kTunedVariant[10][11] = {"] + rows + ["};", "",
+              f"constexpr int kTunedVariant[{N_KERNELS}][11] = {{"] + rows + ["};", "",
               "constexpr int tuned_variant(int kernel, int n) {",
               "  for (int l = 0; l < 11; ++l)",
-              "    if (kTunedLengths[l] == n) return (kernel >= 0 && kernel < 10) ? kTunedVariant[kernel][l] : 0;",
+              "    if (kTunedLengths[l] == n) return (kernel >= 0 && kernel < " + str(N_KERNELS) + ") ? kTunedVariant[kernel][l] : 0;",
               "  return 0;",
               "}", "", "}  // namespace tacaw", ""]
     return "\n".join(lines)
@@ -169,14 +186,30 @@ def main():
         print(json.dumps(measure()))
         return
     results = {}
-    for v in args.variants:
-        env = dict(os.environ, TACAW_NVCC_DEFINES=f"-DTACAW_TUNE_FORCE={v}")
-        r = subprocess.run([sys.executable, "-m", "paper_2602_10064_gb300.tune", "--measure", str(v)], cwd=ROOT,
-                           env=env, capture_output=True, text=True)
-        if r.returncode != 0:
-            raise SystemExit(f"variant {v} failed:\n{r.stdout[-2000:]}\n{r.stderr[-4000:]}")
-        results[v] = json.loads(r.stdout.strip().splitlines()[-1])
-        print(f"variant {v}: " + ", ".join(f"{k} {ms:.2f}" for k, ms in sorted(results[v].items())), flush=True)
+    with tempfile.TemporaryDirectory() as tmp:
+        # one copy of the package per variant, built side by side, measured one after the other
+        def build(v):
+            at = os.path.join(tmp, str(v))
+            for part in ("include", "workloads"):
+                shutil.copytree(os.path.join(ROOT, part), os.path.join(at, part))
+            shutil.copytree(PKG, os.path.join(at, os.path.basename(PKG)),
+                            ignore=shutil.ignore_patterns("_build", "*.so*", "__pycache__"))
+            env = dict(os.environ, TACAW_NVCC_DEFINES=f"-DTACAW_TUNE_FORCE={v}")
+            r = subprocess.run([sys.executable, "-m", "paper_2602_10064_gb300._build"], cwd=at, env=env,
+                               capture_output=True, text=True)
+            if r.returncode != 0:
+                raise SystemExit(f"variant {v} failed:\n{r.stdout[-2000:]}\n{r.stderr[-4000:]}")
+            return at, env
+
+        with cf.ThreadPoolExecutor(max_workers=max(1, (os.cpu_count() or 4) // 2)) as ex:
+            built = list(ex.map(build, args.variants))
+        for v, (at, env) in zip(args.variants, built):
+            r = subprocess.run([sys.executable, "-m", "paper_2602_10064_gb300.tune", "--measure", str(v)], cwd=at,
+                               env=env, capture_output=True, text=True)
+            if r.returncode != 0:
+                raise SystemExit(f"variant {v} failed:\n{r.stdout[-2000:]}\n{r.stderr[-4000:]}")
+            results[v] = json.loads(r.stdout.strip().splitlines()[-1])
+            print(f"variant {v}: " + ", ".join(f"{k} {ms:.3f}" for k, ms in sorted(results[v].items())), flush=True)
     table = choose(results)
     with open(args.out, "w") as fh:
         fh.write(header(table, results))
