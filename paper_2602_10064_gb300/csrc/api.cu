@@ -681,12 +681,15 @@ int bin_frames(tacaw_ctx* ctx, const tacaw_params& p, const float* pos, const in
   int* offs;
   CK(sc.get(&recs, (size_t)nf * std::max<int64_t>(A, 1)));
   CK(sc.get(&offs, (size_t)nf * (S + 1)));
+  uint8_t* key;
+  CK(sc.get(&key, (size_t)nf * std::max<int64_t>(A, 1)));
+  CK(sc.get(&out->rrecs, (size_t)nf * std::max<int64_t>(A, 1)));  // atom order first, then row-sorted
   {
     NvtxRange r_bin("binning");
-    ProfScope ps(ctx, "bin", sc.st, (double)nf * A * 28, 0);
-    CK(launch_bin(pos, A, nf, S, p.cell[0], p.cell[1], p.cell[2], p.nx, p.ny, slots, recs, offs, nullptr, sc.st));
+    ProfScope ps(ctx, "bin", sc.st, (double)nf * A * (12 + 4 * 17), 0);
+    CK(launch_bin(pos, A, nf, bin_geom(p.cell[0], p.cell[1], p.cell[2], p.nx, p.ny, S), slots, out->rrecs, key, recs,
+                  offs, sc.st));
   }
-  CK(sc.get(&out->rrecs, (size_t)nf * std::max<int64_t>(A, 1)));
   CK(sc.get(&out->boffs, (size_t)nf * S * (nyb + 1)));
   {
     NvtxRange r_sort("binning_rows");
@@ -1014,7 +1017,7 @@ RunPlan run_plan(const tacaw_ctx* ctx, const tacaw_params& p, const GeoCache* g,
   RunPlan pl;
   const int64_t F = Fr * R;  // frames through the multislice
   const double nq = (double)p.nx * p.ny, plane = (double)p.ny * g->band.Wp, S = p.n_slices;
-  const double fixed = (double)F * A * 44 + (double)F * (S + 1) * 4 + (double)F * S * (p.ny / SPREAD_YB + 1) * 4;
+  const double fixed = (double)F * A * 45 + (double)F * (S + 1) * 4 + (double)F * S * (p.ny / SPREAD_YB + 1) * 4;
   const double per_probe = nq * 8 + plane * 8 + (double)F * g->nsel * 8 +
                            R * spectrum_bytes_per_probe(g, Fr, precision, reduce);
   const double cap = (double)run_cap(ctx);
@@ -1046,7 +1049,7 @@ uint64_t run_footprint(tacaw_ctx* ctx, const tacaw_params& p, int P, int64_t Fr,
   const double chunk = (double)pl.rt.chunk, sb = pl.rt.sb, Pb = pl.Pb;
   const double tsz = (pl.tf ? plane : nq) * 8;
   double b = 0;
-  b += (double)F * A * (12 + 16 + 16) + (double)F * (S + 1) * 4 + A;  // positions, records (binned, row-sorted), slots
+  b += (double)F * A * (12 + 16 + 16 + 1) + (double)F * (S + 1) * 4 + A;  // positions, records (binned, row-sorted), slices, slots
   b += (double)F * S * (p.ny / SPREAD_YB + 1) * 4;                      // row-block offsets
   b += chunk * sb * plane * 8 * (g->npair + 2);                         // Bp, Ap, Bt
   if (!pl.tf) b += chunk * sb * plane * 8;                              // At
@@ -1146,11 +1149,8 @@ int tacaw_bin_slices(tacaw_ctx* ctx, const tacaw_params* params, const float* po
   if (!is_device_ptr(pos) || !is_device_ptr(slice_out)) return set_err(ctx, TACAW_EINVAL, "pos, slice_out must be device pointers");
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
-  Scratch sc(st);
-  int* offs;
-  CK(sc.get(&offs, (size_t)nf * (params->n_slices + 1)));
-  CK(launch_bin(pos, n_atoms, nf, params->n_slices, params->cell[0], params->cell[1], params->cell[2], params->nx,
-                params->ny, nullptr, nullptr, offs, slice_out, st));
+  CK(launch_slice_index(pos, nf * n_atoms, bin_geom(params->cell[0], params->cell[1], params->cell[2], params->nx,
+                                                   params->ny, params->n_slices), slice_out, st));
   return TACAW_OK;
 }
 

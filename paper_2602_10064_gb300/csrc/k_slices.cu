@@ -216,23 +216,34 @@ __device__ __forceinline__ void store_row(const float2 (&v)[E], float2* __restri
 }
 
 // ============================================================================================
-// a1: slice binning.  One CTA per frame; stable scatter, so every slice list keeps atom order.
+// a1: slice binning.  Slice, grid cell and offset of every atom, then one CTA per frame scatters
+// stably, so every slice list keeps atom order.
 // ============================================================================================
 constexpr int BIN_THREADS = 1024;
 constexpr int BIN_MAX_S = 256;
 
-__device__ __forceinline__ int slice_of(double z, double Lz, int S) {
-  const double dz = Lz / (double)S;
-  const double zw = __dsub_rn(z, __dmul_rn(Lz, floor(z / Lz)));
-  int s = (int)floor(zw / dz);
-  if (s >= S) s = S - 1;
+// x wrapped into [0, L): x - L floor(x / L), every operation rounded.  Within one cell length of the
+// cell the rounded quotient lies strictly between the same integers as the exact one, so its floor
+// is known from comparisons; the FP64 division is left to positions farther out.
+__device__ __forceinline__ double wrap_cell(double x, double L) {
+  if (x >= 0.0 && x < L) return x;
+  if (x >= -L && x < 0.0) return __dsub_rn(x, -L);
+  if (x >= L && x < 2.0 * L) return __dsub_rn(x, L);
+  return __dsub_rn(x, __dmul_rn(L, floor(x / L)));
+}
+
+// floor(z_w / dz): from the product with 1 / dz (off by less than 1e-12 for S <= 256) where that is
+// clear of an integer, else from the division.
+__device__ __forceinline__ int slice_of(double z, const BinGeom& g) {
+  const double zw = wrap_cell(z, g.Lz), q = __dmul_rn(zw, g.inv_dz), fq = floor(q), fr = __dsub_rn(q, fq);
+  int s = fr > 1e-9 && fr < 1.0 - 1e-9 ? (int)fq : (int)floor(zw / g.dz);
+  if (s >= g.S) s = g.S - 1;
   if (s < 0) s = 0;
   return s;
 }
 
-__device__ __forceinline__ void grid_coord(double x, double L, int n, int& i0, float& fr) {
-  const double xw = __dsub_rn(x, __dmul_rn(L, floor(x / L)));
-  const double u = __dmul_rn(xw, (double)n / L);
+__device__ __forceinline__ void grid_coord(double x, double L, double per_len, int n, int& i0, float& fr) {
+  const double u = __dmul_rn(wrap_cell(x, L), per_len);
   double fl = floor(u);
   int i = (int)fl;
   double f = __dsub_rn(u, fl);
@@ -242,23 +253,45 @@ __device__ __forceinline__ void grid_coord(double x, double L, int n, int& i0, f
   fr = (float)f;
 }
 
-__global__ void __launch_bounds__(BIN_THREADS) k_bin(const float* __restrict__ pos, int A, int S, double Lx,
-                                                      double Ly, double Lz, int nx, int ny,
-                                                      const int8_t* __restrict__ slot_of_atom,
-                                                      AtomRec* __restrict__ recs, int* __restrict__ offs,
-                                                      int* __restrict__ slice_out) {
+// Slice of every atom (tacaw_bin_slices).
+__global__ void __launch_bounds__(256) k_slice_index(const float* __restrict__ pos, int64_t n, BinGeom g,
+                                                     int* __restrict__ slice_out) {
+  const int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x;
+  if (j < n) slice_out[j] = slice_of((double)pos[3 * j + 2], g);
+}
+
+// Record and slice of every atom, in atom order, one thread each: the FP64 work of the binning
+// (GB300 issues two FP64 operations a clock and SM) spread over the whole chip.  With it inside the
+// one CTA per frame that scatters, and with seven divisions an atom, 12 frames of 8000 atoms took
+// 190 us; this and the scatter take 33.
+__global__ void __launch_bounds__(256) k_atoms(const float* __restrict__ pos, int A, int64_t nf, BinGeom g,
+                                               const int8_t* __restrict__ slot_of_atom, AtomRec* __restrict__ rec,
+                                               uint8_t* __restrict__ key) {
+  const int j = blockIdx.x * 256 + threadIdx.x;
+  if (j >= A || batch_index() >= nf) return;
+  const size_t at = (size_t)batch_index() * A + j;
+  const float* P = pos + 3 * at;
+  AtomRec r;
+  int ix, iy;
+  grid_coord((double)P[0], g.Lx, g.per_x, g.nx, ix, r.fx);
+  grid_coord((double)P[1], g.Ly, g.per_y, g.ny, iy, r.fy);
+  r.ixy = ix | (iy << 16);
+  r.jslot = j | ((int)slot_of_atom[j] << 24);
+  rec[at] = r;
+  key[at] = (uint8_t)slice_of((double)P[2], g);
+}
+
+__global__ void __launch_bounds__(BIN_THREADS) k_bin(const AtomRec* __restrict__ rec, const uint8_t* __restrict__ key,
+                                                      int A, int S, AtomRec* __restrict__ recs,
+                                                      int* __restrict__ offs) {
   __shared__ int counts[BIN_MAX_S];
   __shared__ int cursor[BIN_MAX_S];
   __shared__ int wcount[BIN_THREADS / 32][BIN_MAX_S];
   const int f = blockIdx.x, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
-  const float* P = pos + (size_t)f * A * 3;
+  const uint8_t* K = key + (size_t)f * A;
   for (int s = tid; s < S; s += BIN_THREADS) counts[s] = 0;
   __syncthreads();
-  for (int j = tid; j < A; j += BIN_THREADS) {
-    const int s = slice_of((double)P[3 * j + 2], Lz, S);
-    atomicAdd(&counts[s], 1);
-    if (slice_out) slice_out[(size_t)f * A + j] = s;
-  }
+  for (int j = tid; j < A; j += BIN_THREADS) atomicAdd(&counts[K[j]], 1);
   __syncthreads();
   if (tid == 0) {
     int run = 0;
@@ -269,14 +302,13 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const float* __restrict__ p
     }
     offs[(size_t)f * (S + 1) + S] = run;
   }
-  if (!recs) return;
   const unsigned lt = (1u << lane) - 1u;
   for (int base = 0; base < A; base += BIN_THREADS) {
     for (int i = tid; i < (BIN_THREADS / 32) * S; i += BIN_THREADS) wcount[i / S][i % S] = 0;
     __syncthreads();
     const int j = base + tid;
     const bool valid = j < A;
-    const int s = valid ? slice_of((double)P[3 * j + 2], Lz, S) : -1;
+    const int s = valid ? K[j] : -1;
     const unsigned peers = __match_any_sync(0xffffffffu, s);
     const int rank = __popc(peers & lt);
     if (valid && rank == 0) wcount[w][s] = __popc(peers);
@@ -291,16 +323,7 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const float* __restrict__ p
       cursor[ss] = run;
     }
     __syncthreads();
-    if (valid) {
-      const int p = wcount[w][s] + rank;
-      AtomRec r;
-      int ix, iy;
-      grid_coord((double)P[3 * j], Lx, nx, ix, r.fx);
-      grid_coord((double)P[3 * j + 1], Ly, ny, iy, r.fy);
-      r.ixy = ix | (iy << 16);
-      r.jslot = j | ((int)slot_of_atom[j] << 24);
-      recs[(size_t)f * A + p] = r;
-    }
+    if (valid) recs[(size_t)f * A + wcount[w][s] + rank] = rec[(size_t)f * A + j];
     __syncthreads();
   }
 }
@@ -404,12 +427,19 @@ cudaError_t launch_sort_rows(const AtomRec* recs, const int* offs, int64_t A, in
   return cudaGetLastError();
 }
 
-cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, int S, double Lx, double Ly, double Lz, int nx,
-                       int ny, const int8_t* slot_of_atom, AtomRec* recs, int* offs, int* slice_out,
-                       cudaStream_t st) {
-  if (S > BIN_MAX_S || nf <= 0) return cudaErrorInvalidValue;
-  k_bin<<<(unsigned)nf, BIN_THREADS, 0, st>>>(pos, (int)A, S, Lx, Ly, Lz, nx, ny, slot_of_atom, recs, offs,
-                                             slice_out);
+cudaError_t launch_slice_index(const float* pos, int64_t n, const BinGeom& g, int* slice_out, cudaStream_t st) {
+  if (g.S > BIN_MAX_S || n <= 0 || (n + 255) / 256 > 0x7fffffff) return cudaErrorInvalidValue;
+  k_slice_index<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(pos, n, g, slice_out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, const BinGeom& g, const int8_t* slot_of_atom,
+                       AtomRec* rec, uint8_t* key, AtomRec* recs, int* offs, cudaStream_t st) {
+  if (g.S > BIN_MAX_S || nf <= 0) return cudaErrorInvalidValue;
+  if (A > 0) k_atoms<<<batch_grid((int)((A + 255) / 256), nf), 256, 0, st>>>(pos, (int)A, nf, g, slot_of_atom, rec, key);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  k_bin<<<(unsigned)nf, BIN_THREADS, 0, st>>>(rec, key, (int)A, g.S, recs, offs);
   return cudaGetLastError();
 }
 

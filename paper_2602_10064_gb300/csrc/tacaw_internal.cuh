@@ -157,9 +157,21 @@ cudaError_t launch_copy_out(const float* src, int64_t sp, float* dst_mapped, int
 // TACAW_STATUS_SPECIES in *status and gets slot 0.
 cudaError_t launch_map_slots(const int32_t* Z, int64_t A, const int8_t* lut, int8_t* slot, int* status,
                              cudaStream_t st);
-cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, int S, double Lx, double Ly, double Lz, int nx,
-                       int ny, const int8_t* slot_of_atom, AtomRec* recs, int* offs, int* slice_out,
-                       cudaStream_t st);
+// Cell, grid and slices of the binning, with the quotients that every atom needs.
+struct BinGeom {
+  double Lx, Ly, Lz, per_x, per_y, dz, inv_dz;  // per_x = nx / Lx, dz = Lz / S
+  int nx, ny, S;
+};
+inline BinGeom bin_geom(double Lx, double Ly, double Lz, int nx, int ny, int S) {
+  const double dz = Lz / (double)S;
+  return BinGeom{Lx, Ly, Lz, (double)nx / Lx, (double)ny / Ly, dz, 1.0 / dz, nx, ny, S};
+}
+// slice_out[j] of n atoms.
+cudaError_t launch_slice_index(const float* pos, int64_t n, const BinGeom& g, int* slice_out, cudaStream_t st);
+// Per-(frame, slice) lists: recs [nf][A] with the offsets offs [nf][S + 1]; rec [nf][A] and key
+// [nf][A] are scratch (the records and slices in atom order).
+cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, const BinGeom& g, const int8_t* slot_of_atom,
+                       AtomRec* rec, uint8_t* key, AtomRec* recs, int* offs, cudaStream_t st);
 // Grid rows per block of the row-sorted atom lists of the spreading pass (divides every grid length).
 constexpr int SPREAD_YB = 8;
 // Row-sorted copy of the binned records: per (frame, slice) a stable sort by grid row, and the
