@@ -86,7 +86,7 @@ void gauss_legendre(int n, std::vector<double>& x, std::vector<double>& w) {
   }
 }
 
-constexpr int kSpreadHalf = 6;         // kernel width w = 12 grid points
+constexpr int kSpreadHalf = SPREAD_HALF;  // kernel width w = 12 grid points
 constexpr double kSpreadBeta = 24.0;   // beta = 2.0 w
 
 double es_phi(double z) {
@@ -705,7 +705,6 @@ int potential_block(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const Bi
                     int nfc, int s0, int sbc, float2* Bp, float2* Ap, cudaStream_t st) {
   const int S = p.n_slices, ny = p.ny, nyb = ny / SPREAD_YB, nfs = nfc * sbc;
   const Geo geo{p.nx, p.ny, ctx->tw};
-  const SpreadKernel sk{kSpreadHalf, (float)kSpreadBeta};
   const double W8 = (double)g->band.W * 8.0, fx = 5.0 * p.nx * std::log2((double)p.nx),
                fy = 5.0 * ny * std::log2((double)ny);
   NvtxRange r_pot("potential");
@@ -713,7 +712,7 @@ int potential_block(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const Bi
     ProfScope ps(ctx, "splat_row", st, (double)nfc * A * 16 * sbc / S + (double)nfs * g->npair * ny * W8,
                  (double)nfs * g->npair * ny * fx);
     CK(launch_splat_row(geo, g->band, bn.rrecs + (size_t)f0 * A, bn.boffs + (size_t)f0 * S * (nyb + 1), A, S, s0,
-                        sbc, nfs, g->npair, sk, Bp, (int)ctx->static_band, st));
+                        sbc, nfs, g->npair, (float)kSpreadBeta, Bp, (int)ctx->static_band, st));
   }
   {
     ProfScope ps(ctx, "col_pot", st, (double)nfs * (g->npair + 1) * ny * W8 + (double)g->npair * ny * W8,

@@ -138,10 +138,8 @@ __device__ __forceinline__ int band_x_col(const Band& b, int nx, int x) {
 }
 
 // ---- host launchers (k_slices.cu) ---------------------------------------------------------
-struct SpreadKernel {
-  int half;    // h = w / 2 grid points
-  float beta;  // exp(beta (sqrt(1 - z^2) - 1))
-};
+// Spreading kernel exp(beta (sqrt(1 - z^2) - 1)) over z = d / SPREAD_HALF: 2 SPREAD_HALF grid points.
+constexpr int SPREAD_HALF = 6;
 
 // Bits of the context's device status word, read and cleared by tacaw_check.
 constexpr int TACAW_STATUS_TIMEOUT = 1;  // a kernel's bounded wait ran out
@@ -182,7 +180,7 @@ cudaError_t launch_sort_rows(const AtomRec* recs, const int* offs, int64_t A, in
 // Spreading row pass of slices [s0, s0 + sb) of nfs / sb frames (batch = (frame, slice, pair)),
 // from the row-sorted records and their row-block offsets.
 cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A, int S,
-                             int s0, int sb, int nfs, int npair, SpreadKernel sk, float2* Bp, int static_band,
+                             int s0, int sb, int nfs, int npair, float beta, float2* Bp, int static_band,
                              cudaStream_t st);
 cudaError_t launch_col_pot(const Geo& g, const Band& b, const float2* Bp, const float2* mtab, int npair, int nfs,
                            float2* Ap, int static_band, cudaStream_t st);
