@@ -594,6 +594,8 @@ int tacaw_destroy(tacaw_ctx* ctx) {
   cudaDeviceSynchronize();
   for (auto& sp : ctx->staging.inflight) cudaEventDestroy(sp.done);
   for (cudaEvent_t ev : ctx->staging.free_events) cudaEventDestroy(ev);
+  if (ctx->species_event) cudaEventDestroy(ctx->species_event);
+  if (ctx->species_flag) cudaFreeHost(ctx->species_flag);
   if (ctx->staging.base) cudaFreeHost(ctx->staging.base);
   for (void* p : ctx->owned) cudaFree(p);
   delete ctx;
@@ -631,33 +633,40 @@ int tacaw_load_form_factors(tacaw_ctx* ctx, const int32_t* Z, const double* coef
 
 namespace tacaw {
 
-// Slot (form-factor table index) of every atom; host Z in, device int8 out.
-// Form-factor slot of every atom.  Z on the device with device_check: mapped on the device, an
-// unknown species reported through the status word (tacaw_check), so the host never waits
-// for the stream.  Otherwise Z is checked on the host and an unknown species is EINVAL here.
+// Form-factor slot of every atom.  Z on the device is mapped there; what becomes of an unknown
+// species depends on the caller: device_check reports it through the context's status word
+// (tacaw_check), else through a flag of this call that species_verdict reads once the call's work is
+// enqueued, so the device does not wait for the host either way.  Z on the host is checked here
+// (EINVAL).
 int make_slots(tacaw_ctx* ctx, const int32_t* Z, int64_t A, bool z_on_device, bool device_check, Scratch& sc,
                int8_t** d_slot) {
-  if (z_on_device && device_check) {
+  if (z_on_device) {
     CK(sc.get(d_slot, std::max<int64_t>(A, 1)));
-    ProfScope ps(ctx, "map_slots", sc.st, (double)A * 5, 0);
-    CK(launch_map_slots(Z, A, ctx->d_zslot, *d_slot, ctx->d_status, sc.st));
-    return TACAW_OK;
-  }
-  std::vector<int32_t> hz(A);
-  if (A > 0) {
-    if (z_on_device) {
-      CK(cudaMemcpyAsync(hz.data(), Z, sizeof(int32_t) * A, cudaMemcpyDeviceToHost, sc.st));
-      CK(cudaStreamSynchronize(sc.st));
-    } else {
-      std::memcpy(hz.data(), Z, sizeof(int32_t) * A);
+    int* bad = ctx->d_status;
+    if (!device_check) {
+      if (!ctx->species_flag) {
+        CK(cudaEventCreateWithFlags(&ctx->species_event, cudaEventDisableTiming));
+        CK(cudaMallocHost((void**)&ctx->species_flag, sizeof(int)));
+      }
+      CK(sc.get(&bad, 1));
+      CK(cudaMemsetAsync(bad, 0, sizeof(int), sc.st));
     }
+    {
+      ProfScope ps(ctx, "map_slots", sc.st, (double)A * 5, 0);
+      CK(launch_map_slots(Z, A, ctx->d_zslot, *d_slot, bad, sc.st));
+    }
+    if (!device_check) {
+      CK(cudaMemcpyAsync(ctx->species_flag, bad, sizeof(int), cudaMemcpyDeviceToHost, sc.st));
+      CK(cudaEventRecord(ctx->species_event, sc.st));
+    }
+    return TACAW_OK;
   }
   std::vector<int8_t> hs(A);
   for (int64_t j = 0; j < A; ++j) {
     int s = -1;
     for (size_t i = 0; i < ctx->ffZ.size(); ++i)
-      if (ctx->ffZ[i] == hz[j]) s = (int)i;
-    if (s < 0) return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, hz[j]);
+      if (ctx->ffZ[i] == Z[j]) s = (int)i;
+    if (s < 0) return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, Z[j]);
     hs[j] = (int8_t)s;
   }
   CK(sc.get(d_slot, A));
@@ -666,6 +675,19 @@ int make_slots(tacaw_ctx* ctx, const int32_t* Z, int64_t A, bool z_on_device, bo
     CK(staged_copy(ctx, *d_slot, hs.data(), A, sc.st));
   }
   return TACAW_OK;
+}
+
+// Result of the species check of make_slots without device_check: waits for the mapping only.
+int species_verdict(tacaw_ctx* ctx, const int32_t* Z, int64_t A, cudaStream_t st) {
+  CK(cudaEventSynchronize(ctx->species_event));
+  if (!*ctx->species_flag) return TACAW_OK;
+  std::vector<int32_t> hz(A);
+  CK(cudaMemcpyAsync(hz.data(), Z, sizeof(int32_t) * A, cudaMemcpyDeviceToHost, st));
+  CK(cudaStreamSynchronize(st));
+  for (int64_t j = 0; j < A; ++j)
+    if (std::find(ctx->ffZ.begin(), ctx->ffZ.end(), hz[j]) == ctx->ffZ.end())
+      return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, hz[j]);
+  return set_err(ctx, TACAW_EINVAL, "an atom's Z is not in the form-factor table");
 }
 
 // Binned atoms of frames [0, nf): per-(frame, slice) lists, then the row-sorted copy with the
@@ -823,50 +845,32 @@ int build_probes(tacaw_ctx* ctx, const tacaw_params& p, const tacaw_probe& pr, S
   if (W == 0) return set_err(ctx, TACAW_EINVAL, "probe aperture holds no k point");
   int64_t count = 0;
   for (int c = 0; c < W; ++c) count += nb[c] < 0 ? 0 : (nb[c] >= ny / 2 ? ny : 2 * nb[c] + 1);
-  std::vector<float2> ex((size_t)P * Wp, make_float2(0.f, 0.f)), ey((size_t)P * ny);
-  for (int ip = 0; ip < P; ++ip) {
-    const double xp = pr.xy ? pr.xy[2 * ip] : 0.0, yp = pr.xy ? pr.xy[2 * ip + 1] : 0.0;
-    for (int c = 0; c < W; ++c) {
-      const int x = c <= mb ? c : nx - (W - c);
-      const double a = -2.0 * M_PI * kfreq(x, nx, Lx) * xp;
-      ex[(size_t)ip * Wp + c] = make_float2((float)std::cos(a), (float)std::sin(a));
-    }
-    for (int y = 0; y < ny; ++y) {
-      const double a = -2.0 * M_PI * kfreq(y, ny, Ly) * yp;
-      ey[(size_t)ip * ny + y] = make_float2((float)std::cos(a), (float)std::sin(a));
-    }
-  }
-  // aberration phase exp(-i chi(k)) over the aperture columns, FP64 on the host
-  std::vector<float2> chi;
-  if (has_aberrations(pr)) {
-    const double lam = wavelength_A(p.voltage_ev), cs = pr.cs_mm * 1e7;
-    chi.assign((size_t)ny * Wp, make_float2(0.f, 0.f));
-    for (int c = 0; c < W; ++c) {
-      const int x = c <= mb ? c : nx - (W - c);
-      const double kx = kfreq(x, nx, Lx);
-      for (int y = 0; y < ny; ++y) {
-        const double ky = kfreq(y, ny, Ly), k2 = kx * kx + ky * ky, phk = std::atan2(ky, kx);
-        const double ph = M_PI * lam * k2 * (pr.defocus + pr.astig * std::cos(2.0 * (phk - pr.astig_angle))) +
-                          (2.0 * M_PI / 3.0) * pr.coma * lam * lam * k2 * std::sqrt(k2) * std::cos(phk - pr.coma_angle) +
-                          0.5 * M_PI * cs * lam * lam * lam * k2 * k2;
-        chi[(size_t)y * Wp + c] = make_float2((float)std::cos(ph), (float)-std::sin(ph));
-      }
-    }
-  }
+  const double lam = wavelength_A(p.voltage_ev);
+  ProbeTables tab{nx, ny, W, Wp, mb, P, Lx, Ly};
+  tab.c1 = lam * pr.defocus;
+  tab.a_cos = lam * pr.astig * std::cos(2.0 * pr.astig_angle);
+  tab.a_sin = lam * pr.astig * std::sin(2.0 * pr.astig_angle);
+  tab.b_cos = (2.0 / 3.0) * pr.coma * lam * lam * std::cos(pr.coma_angle);
+  tab.b_sin = (2.0 / 3.0) * pr.coma * lam * lam * std::sin(pr.coma_angle);
+  tab.c3 = 0.5 * pr.cs_mm * 1e7 * lam * lam * lam;
   int* d_nb;
+  double* d_xy = nullptr;
   float2 *d_ex, *d_ey, *Bpr, *d_chi = nullptr;
-  if (!chi.empty()) {
-    CK(sc.get(&d_chi, chi.size()));
-    CK(staged_copy(ctx, d_chi, chi.data(), sizeof(float2) * chi.size(), sc.st));
-  }
+  if (has_aberrations(pr)) CK(sc.get(&d_chi, (size_t)ny * Wp));
   CK(sc.get(&d_nb, Wp));
-  CK(sc.get(&d_ex, ex.size()));
-  CK(sc.get(&d_ey, ey.size()));
+  CK(sc.get(&d_ex, (size_t)P * Wp));
+  CK(sc.get(&d_ey, (size_t)P * ny));
   CK(sc.get(&Bpr, (size_t)P * ny * Wp));
   CK(sc.get(psi0, (size_t)P * ny * nx));
   CK(staged_copy(ctx, d_nb, nb.data(), sizeof(int) * Wp, sc.st));
-  CK(staged_copy(ctx, d_ex, ex.data(), sizeof(float2) * ex.size(), sc.st));
-  CK(staged_copy(ctx, d_ey, ey.data(), sizeof(float2) * ey.size(), sc.st));
+  if (pr.xy) {
+    CK(sc.get(&d_xy, 2 * (size_t)P));
+    CK(staged_copy(ctx, d_xy, pr.xy, sizeof(double) * 2 * P, sc.st));
+  }
+  {
+    ProfScope ps(ctx, "probe_tables", sc.st, 8.0 * ((double)P * (Wp + ny) + (d_chi ? (double)ny * Wp : 0.0)), 0);
+    CK(launch_probe_tables(tab, d_xy, d_nb, d_ex, d_ey, d_chi, sc.st));
+  }
   const Band ap{W, Wp, mb, d_nb};
   const Geo geo{nx, ny, ctx->tw};
   {
@@ -1175,12 +1179,15 @@ int tacaw_build_potential(tacaw_ctx* ctx, const tacaw_params* params, const floa
   const Geo geo{p.nx, p.ny, ctx->tw};
   const size_t plane = (size_t)p.ny * g->band.Wp;
   const int64_t chunk = chunk_frames(nf, p.n_slices * plane * 8 * (g->npair + 1), (size_t)1 << 30);
-  return potential_chunks(ctx, p, g, pos, slots, n_atoms, nf, chunk, p.n_slices, sc,
+  TRY_RC(potential_chunks(ctx, p, g, pos, slots, n_atoms, nf, chunk, p.n_slices, sc,
                           [&](int64_t f0, int nfc, int, int, float2* Ap) {
+    ProfScope ps(ctx, "row_pot_out", st, (double)nfc * p.n_slices * p.ny * (8.0 * g->band.W + 4.0 * p.nx),
+                 (double)nfc * p.n_slices * p.ny * 5.0 * p.nx * std::log2((double)p.nx));
     CK(launch_row_pot_out(geo, g->band, Ap, nfc * p.n_slices, 0, 0.f,
                           V_out + (size_t)f0 * p.n_slices * p.ny * p.nx, nullptr, (int)ctx->static_band, st));
     return TACAW_OK;
-  });
+  }));
+  return species_verdict(ctx, Z, n_atoms, st);
 }
 
 int tacaw_transmission(tacaw_ctx* ctx, const tacaw_params* params, const float* V, int64_t nf, float* t_out,

@@ -785,6 +785,54 @@ __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, N
 // ============================================================================================
 // Probe: psi0(k) = A(k) exp(-2 pi i k.r_p) amp, then a unitary inverse transform.
 // ============================================================================================
+// Phase tables of P probes, FP64 rounded to float: ex [P][Wp] and ey [P][ny], exp(-2 pi i k x_p) over
+// the aperture columns and the rows, and chi [ny][Wp] (if any), exp(-i chi(k)).  The angular terms of
+// chi are polynomials in (kx, ky): k^2 cos 2(phi - a) = (kx^2 - ky^2) cos 2a + 2 kx ky sin 2a and
+// k cos(phi - a) = kx cos a + ky sin a.  On the host these tables were most of a call: 37 aberrated
+// probes at 384^2 1.4 ms before the first launch.
+__global__ void __launch_bounds__(256) k_probe_tables(ProbeTables q, const double* __restrict__ xy,
+                                                      const int* __restrict__ nb, float2* __restrict__ ex,
+                                                      float2* __restrict__ ey, float2* __restrict__ chi) {
+  const int64_t nex = (int64_t)q.P * q.Wp, ney = (int64_t)q.P * q.ny, nchi = chi ? (int64_t)q.ny * q.Wp : 0;
+  for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < nex + ney + nchi; i += (int64_t)gridDim.x * 256) {
+    double s, c;
+    if (i < nex) {
+      const int p = (int)(i / q.Wp), cc = (int)(i - (int64_t)p * q.Wp);
+      float2 v = make_float2(0.f, 0.f);
+      if (cc < q.W) {
+        sincospi(-2.0 * ((double)q.freq_x(cc) / q.Lx) * (xy ? xy[2 * p] : 0.0), &s, &c);
+        v = make_float2((float)c, (float)s);
+      }
+      ex[i] = v;
+    } else if (i < nex + ney) {
+      const int64_t k = i - nex;
+      const int p = (int)(k / q.ny), y = (int)(k - (int64_t)p * q.ny);
+      sincospi(-2.0 * ((double)fftfreq_index(y, q.ny) / q.Ly) * (xy ? xy[2 * p + 1] : 0.0), &s, &c);
+      ey[k] = make_float2((float)c, (float)s);
+    } else {
+      const int64_t k = i - nex - ney;
+      const int y = (int)(k / q.Wp), cc = (int)(k - (int64_t)y * q.Wp), n = fftfreq_index(y, q.ny);
+      float2 v = make_float2(0.f, 0.f);
+      if (cc < q.W && abs(n) <= nb[cc]) {
+        const double kx = (double)q.freq_x(cc) / q.Lx, ky = (double)n / q.Ly, k2 = kx * kx + ky * ky;
+        // chi / pi
+        const double h = q.c1 * k2 + q.a_cos * (kx * kx - ky * ky) + q.a_sin * (2.0 * kx * ky) +
+                         k2 * (q.b_cos * kx + q.b_sin * ky) + q.c3 * k2 * k2;
+        sincospi(-h, &s, &c);
+        v = make_float2((float)c, (float)s);
+      }
+      chi[k] = v;
+    }
+  }
+}
+
+cudaError_t launch_probe_tables(const ProbeTables& q, const double* xy, const int* nb, float2* ex, float2* ey,
+                                float2* chi, cudaStream_t st) {
+  const int64_t n = (int64_t)q.P * (q.Wp + q.ny) + (chi ? (int64_t)q.ny * q.Wp : 0);
+  k_probe_tables<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(q, xy, nb, ex, ey, chi);
+  return cudaGetLastError();
+}
+
 template <int NY>
 __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL, NY, ProbeColCfg<NY>>())
     k_probe_col(Geo geo, Band ap, const float2* __restrict__ ex, const float2* __restrict__ ey,

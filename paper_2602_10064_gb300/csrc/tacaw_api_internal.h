@@ -90,6 +90,8 @@ struct tacaw_ctx {
   std::map<int64_t, float2*> time_tw;
   std::map<int64_t, std::pair<float2*, float2*>> chirps;  // chirp-z tables (chirp, spectrum) per F
   std::map<int64_t, std::pair<void*, void*>> dft_ops;  // tensor-core DFT operands (hi, lo) per F and kind
+  int* species_flag = nullptr;  // page-locked: the species check of tacaw_build_potential
+  cudaEvent_t species_event = nullptr;
   int* d_status = nullptr;  // device status word: bits TACAW_STATUS_* (tacaw_internal.cuh)
   int64_t max_chunk_frames = 0;  // option: cap on frames per chunk (0 = automatic)
   int64_t max_slice_block = 0;   // option: cap on slices per block of a run (0 = automatic)

@@ -194,6 +194,19 @@ cudaError_t launch_row_vt(const Geo& g, const Band& b, const float* V, int nfs, 
 cudaError_t launch_col_t(const Geo& g, const Band& b, const float2* Bt, int nfs, float scale, float2* At,
                          int static_band, cudaStream_t st);
 cudaError_t launch_row_tout(const Geo& g, const Band& b, const float2* At, int nfs, float2* t, cudaStream_t st);
+// Phase tables of P probes over the aperture columns W (padded Wp, FFT order with mb non-negative
+// frequencies first), and the coefficients of chi / pi:
+// c1 k^2 + a_cos (kx^2 - ky^2) + a_sin 2 kx ky + k^2 (b_cos kx + b_sin ky) + c3 k^4.
+struct ProbeTables {
+  int nx, ny, W, Wp, mb, P;
+  double Lx, Ly, c1, a_cos, a_sin, b_cos, b_sin, c3;
+  __host__ __device__ int freq_x(int c) const {
+    const int x = c <= mb ? c : nx - (W - c);
+    return x < (nx + 1) / 2 ? x : x - nx;
+  }
+};
+cudaError_t launch_probe_tables(const ProbeTables& q, const double* xy, const int* nb, float2* ex, float2* ey,
+                                float2* chi, cudaStream_t st);
 // chi (nullable): exp(-i chi(k)) over [ny][ap.Wp]
 cudaError_t launch_probe_col(const Geo& g, const Band& ap, const float2* ex, const float2* ey, const float2* chi,
                              int P, float amp, float2* Bpr, cudaStream_t st);
