@@ -311,13 +311,13 @@ struct GroupSync {
   }
 };
 
-// Shared-memory padding: one slot per 2^SH elements along the transform.  The first pass of every
-// plan stores each thread's R1 outputs contiguously (stride R1 across the threads of a warp); the pad
-// makes that stride odd, so that those 64-bit stores, and the own-position reads of every pass, stay
-// at (or near) the minimum two wavefronts per warp.
+// Shared-memory padding: one slot per 2^SH elements along the transform, for the fewest wavefronts
+// of a plan's exchanges counted over the threads of a warp (64-bit accesses, 16 lanes a wavefront at
+// best): the minimum for the powers of two, 96 and 192; 240 of at least 192 for 384 and 768, 256 of
+// 192 for 1152.
 template <int N, int E>
 struct PadShift {
-  static constexpr int SH = E == 24 ? (N == 96 ? 2 : N == 1152 ? 4 : 3) : (E == 8 || N <= 64) ? 3 : (E == 32 ? 5 : 4);
+  static constexpr int SH = N == 96 ? 2 : (N == 192 || E == 8 || N <= 64) ? 3 : (E == 32 ? 5 : 4);
 };
 template <int N, int E>
 struct RowIdx {
@@ -326,7 +326,7 @@ struct RowIdx {
   __device__ __forceinline__ int operator()(int x) const { return base + x + (x >> SH); }
 };
 template <int N, int E>
-__host__ __device__ constexpr int row_smem_stride() { return N + (N >> PadShift<N, E>::SH); }
+__host__ __device__ constexpr int row_smem_stride() { return N + (N >> PadShift<N, E>::SH) + (N == 96 ? 4 : 0); }
 
 // Column-owned transforms: C columns interleaved in shared memory, column c fastest, padded
 // with one row of C slots per 2^SH rows (SH = 0: unpadded); the threads of one transform are

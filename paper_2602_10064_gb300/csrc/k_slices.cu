@@ -90,7 +90,8 @@ struct ColCfg {
   static constexpr int C0 = ((TARGET / 2) << WIDE) / T;
   static constexpr int C = C0 > 32 ? 32 : (C0 < 4 ? 4 : floor_pow2(C0));  // columns per CTA (divides Wp)
   static constexpr int THREADS = C * T;
-  // padding of the interleaved columns: measured to pay only with 32 elements per thread
+  // padding of the interleaved columns: pays only with 32 elements per thread (with 8 columns of 1152
+  // points it saves 20% of the exchanges' wavefronts, but the pass takes 264 us instead of 218)
   static constexpr int SH = E == 32 ? 5 : 0;
   static constexpr int SMEM = (N + (SH ? (N >> SH) : 0)) * C * (int)sizeof(float2);
 };
