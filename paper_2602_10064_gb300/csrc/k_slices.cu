@@ -569,13 +569,12 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
     //    128 slices 117 us, this 99.
     int c0 = 0, c1 = total;
     if (!whole) {
-      constexpr int RPW = T < 32 ? 32 / T : 1;  // rows of a warp
-      const int g0 = T < 32 ? (tid / 32) * RPW : g, lane = tid & 31;
+      const int lane = tid & 31, g0 = (tid - lane) / T, g1 = (tid - lane + 31) / T;  // rows of this warp
       c1 = 0;
       for (int c = 0; c < total; c += 32) {
         const int r = c + lane < total ? crow[c + lane] : ny;
         c0 += __popc(__ballot_sync(0xffffffffu, r < g0 - h));
-        c1 += __popc(__ballot_sync(0xffffffffu, r <= g0 + RPW - 2 + h));
+        c1 += __popc(__ballot_sync(0xffffffffu, r <= g1 - 1 + h));
       }
     }
     float* arow = reinterpret_cast<float*>(acc + g * NX);
