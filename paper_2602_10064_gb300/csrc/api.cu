@@ -722,31 +722,41 @@ int bin_frames(tacaw_ctx* ctx, const tacaw_params& p, const float* pos, const in
 }
 
 // Potential of slices [s0, s0 + sbc) of frames [f0, f0 + nfc): the spreading row pass into Bp
-// and the column pass into Ap [nfc][sbc][ny][Wp] (compact columns), for a row pass out of it.
+// and the column pass into Ap, for a row pass out of it: a plane [ny][Wp] (compact columns) per slice,
+// or, with one species loaded, per pair of slices.  The pairs are fixed (2i, 2i + 1), so a slice's
+// bits do not depend on the blocks: one cut by a block is formed by both of its blocks.
+struct PotPlanes {
+  const float2* Ap;
+  int planes;           // in all
+  tacaw::SlicePairs sp;
+};
 int potential_block(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const Binned& bn, int64_t A, int64_t f0,
-                    int nfc, int s0, int sbc, float2* Bp, float2* Ap, cudaStream_t st) {
-  const int S = p.n_slices, ny = p.ny, nyb = ny / SPREAD_YB, nfs = nfc * sbc;
+                    int nfc, int s0, int sbc, float2* Bp, float2* Ap, cudaStream_t st, PotPlanes* out) {
+  const int S = p.n_slices, ny = p.ny, nyb = ny / SPREAD_YB, two = g->nslot == 1;
+  const int per_frame = two ? (s0 + sbc - 1) / 2 - s0 / 2 + 1 : sbc, planes = nfc * per_frame;
+  const int* boffs = bn.boffs + (size_t)f0 * S * (nyb + 1);
   const Geo geo{p.nx, p.ny, ctx->tw};
   const double W8 = (double)g->band.W * 8.0, fx = 5.0 * p.nx * std::log2((double)p.nx),
                fy = 5.0 * ny * std::log2((double)ny);
   NvtxRange r_pot("potential");
   {
-    ProfScope ps(ctx, "splat_row", st, (double)nfc * A * 16 * sbc / S + (double)nfs * g->npair * ny * W8,
-                 (double)nfs * g->npair * ny * fx);
-    CK(launch_splat_row(geo, g->band, bn.rrecs + (size_t)f0 * A, bn.boffs + (size_t)f0 * S * (nyb + 1), A, S, s0,
-                        sbc, nfs, g->npair, (float)kSpreadBeta, Bp, (int)ctx->static_band, st));
+    ProfScope ps(ctx, "splat_row", st, (double)nfc * A * 16 * sbc / S + (double)planes * g->npair * ny * W8,
+                 (double)planes * g->npair * ny * fx);
+    CK(launch_splat_row(geo, g->band, bn.rrecs + (size_t)f0 * A, boffs, A, S, s0, per_frame, planes, g->npair, two,
+                        (float)kSpreadBeta, Bp, (int)ctx->static_band, st));
   }
   {
-    ProfScope ps(ctx, "col_pot", st, (double)nfs * (g->npair + 1) * ny * W8 + (double)g->npair * ny * W8,
-                 (double)nfs * (g->npair + 1) * g->band.W * fy);
-    CK(launch_col_pot(geo, g->band, Bp, g->mtab, g->npair, nfs, Ap, (int)ctx->static_band, st));
+    ProfScope ps(ctx, "col_pot", st, (double)planes * (g->npair + 1) * ny * W8 + (double)g->npair * ny * W8,
+                 (double)planes * (g->npair + 1) * g->band.W * fy);
+    CK(launch_col_pot(geo, g->band, Bp, g->mtab, g->npair, planes, Ap, (int)ctx->static_band, st));
   }
+  *out = PotPlanes{Ap, planes, tacaw::SlicePairs{two ? per_frame : 0, S, s0, sbc, boffs}};
   return TACAW_OK;
 }
 
 // Potential of frames [0, nf): binning, then per chunk of `chunk` frames and per block of `sb`
-// slices the spreading row pass and the column pass.  Leaves Ap [nfc][sbc][ny][Wp] to
-// `sink(f0, nfc, s0, sbc, Ap)`, which runs the row pass out of the potential.
+// slices the spreading row pass and the column pass.  Leaves the planes to `sink(f0, nfc, planes)`,
+// which runs the row pass out of the potential.
 template <class Sink>
 int potential_chunks(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const float* pos, const int8_t* slots,
                      int64_t A, int64_t nf, int64_t chunk, int sb, Scratch& sc, Sink sink) {
@@ -761,8 +771,9 @@ int potential_chunks(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const f
     const int nfc = (int)std::min<int64_t>(chunk, nf - f0);
     for (int s0 = 0; s0 < S; s0 += sb) {
       const int sbc = std::min(sb, S - s0);
-      TRY_RC(potential_block(ctx, p, g, bn, A, f0, nfc, s0, sbc, Bp, Ap, sc.st));
-      TRY_RC(sink(f0, nfc, s0, sbc, Ap));
+      PotPlanes pp;
+      TRY_RC(potential_block(ctx, p, g, bn, A, f0, nfc, s0, sbc, Bp, Ap, sc.st, &pp));
+      TRY_RC(sink(f0, nfc, pp));
     }
   }
   return TACAW_OK;
@@ -774,7 +785,7 @@ int64_t chunk_frames(int64_t nf, size_t per_frame, size_t cap) {
   return std::min<int64_t>(c, nf);
 }
 
-// Band-limited transmission of nfs slices from Ap (potential column-pass output) or V.
+// Band-limited transmission of nfs slices from the potential's planes or from V.
 // With `compact` (and the transmission band limit on) it stops after the column pass and
 // leaves the compact At [nfs][ny][Wp] in t, for the fused slice row pass; otherwise t is the
 // full [nfs][ny][nx] transmission function.
@@ -796,7 +807,7 @@ int trans_bufs(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, int64_t nfs, 
   return TACAW_OK;
 }
 
-int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const float2* Ap, const float* V, int nfs,
+int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const PotPlanes* pp, const float* V, int nfs,
                       float2* t, Scratch& sc, const TransBufs& tb, bool compact = false) {
   const Geo geo{p.nx, p.ny, ctx->tw};
   const float sig = (float)(sigma_per_VA(p.voltage_ev) / M_PI);  // sincospi takes units of pi
@@ -804,9 +815,9 @@ int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const 
   const double W8 = (double)g->band.W * 8.0, row = (double)nfs * p.ny, fx = 5.0 * p.nx * std::log2((double)p.nx),
                fy = 5.0 * p.ny * std::log2((double)p.ny);
   if (!bl) {
-    if (Ap) {
-      ProfScope ps(ctx, "row_pot_t", sc.st, row * (W8 + 8.0 * p.nx), row * fx);
-      CK(launch_row_pot_out(geo, g->band, Ap, nfs, 2, sig, nullptr, t, (int)ctx->static_band, sc.st));
+    if (pp) {
+      ProfScope ps(ctx, "row_pot_t", sc.st, (double)pp->planes * p.ny * W8 + row * 8.0 * p.nx, (double)pp->planes * p.ny * fx);
+      CK(launch_row_pot_out(geo, g->band, pp->Ap, pp->planes, pp->sp, 2, sig, nullptr, t, (int)ctx->static_band, sc.st));
     } else {
       ProfScope ps(ctx, "row_vt", sc.st, row * 12.0 * p.nx, 0);
       CK(launch_row_vt(geo, g->band, V, nfs, 0, sig, t, sc.st));
@@ -815,9 +826,9 @@ int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const 
   }
   float2* Bt = tb.Bt;
   float2* At = compact ? t : tb.At;
-  if (Ap) {
-    ProfScope ps(ctx, "row_pot_t", sc.st, row * 2 * W8, row * 2 * fx);
-    CK(launch_row_pot_out(geo, g->band, Ap, nfs, 1, sig, nullptr, Bt, (int)ctx->static_band, sc.st));
+  if (pp) {
+    ProfScope ps(ctx, "row_pot_t", sc.st, ((double)pp->planes * p.ny + row) * W8, ((double)pp->planes * p.ny + row) * fx);
+    CK(launch_row_pot_out(geo, g->band, pp->Ap, pp->planes, pp->sp, 1, sig, nullptr, Bt, (int)ctx->static_band, sc.st));
   } else {
     ProfScope ps(ctx, "row_vt", sc.st, row * (4.0 * p.nx + W8), row * fx);
     CK(launch_row_vt(geo, g->band, V, nfs, 1, sig, Bt, sc.st));
@@ -1118,9 +1129,10 @@ int run_impl(tacaw_ctx* ctx, const tacaw_params& p, const tacaw_probe& pr, const
         const int sbc = std::min(rt.sb, S - s0);
         float2* tblk = pl.keep_t ? t + (size_t)f0 * S * tsz : t;
         if (build_t) {
-          TRY_RC(potential_block(ctx, p, g, bn, A, f0, nfc, s0, sbc, Bp, Ap, st));
+          PotPlanes pp;
+          TRY_RC(potential_block(ctx, p, g, bn, A, f0, nfc, s0, sbc, Bp, Ap, st, &pp));
           NvtxRange r("transmission");
-          TRY_RC(transmission_from(ctx, p, g, Ap, nullptr, nfc * sbc, tblk, sc, tb, pl.tf));
+          TRY_RC(transmission_from(ctx, p, g, &pp, nullptr, nfc * sbc, tblk, sc, tb, pl.tf));
         }
         NvtxRange r("multislice");
         if (pl.keep_t)
@@ -1180,10 +1192,11 @@ int tacaw_build_potential(tacaw_ctx* ctx, const tacaw_params* params, const floa
   const size_t plane = (size_t)p.ny * g->band.Wp;
   const int64_t chunk = chunk_frames(nf, p.n_slices * plane * 8 * (g->npair + 1), (size_t)1 << 30);
   TRY_RC(potential_chunks(ctx, p, g, pos, slots, n_atoms, nf, chunk, p.n_slices, sc,
-                          [&](int64_t f0, int nfc, int, int, float2* Ap) {
-    ProfScope ps(ctx, "row_pot_out", st, (double)nfc * p.n_slices * p.ny * (8.0 * g->band.W + 4.0 * p.nx),
-                 (double)nfc * p.n_slices * p.ny * 5.0 * p.nx * std::log2((double)p.nx));
-    CK(launch_row_pot_out(geo, g->band, Ap, nfc * p.n_slices, 0, 0.f,
+                          [&](int64_t f0, int nfc, const PotPlanes& pp) {
+    ProfScope ps(ctx, "row_pot_out", st,
+                 (double)pp.planes * p.ny * 8.0 * g->band.W + (double)nfc * p.n_slices * p.ny * 4.0 * p.nx,
+                 (double)pp.planes * p.ny * 5.0 * p.nx * std::log2((double)p.nx));
+    CK(launch_row_pot_out(geo, g->band, pp.Ap, pp.planes, pp.sp, 0, 0.f,
                           V_out + (size_t)f0 * p.n_slices * p.ny * p.nx, nullptr, (int)ctx->static_band, st));
     return TACAW_OK;
   }));

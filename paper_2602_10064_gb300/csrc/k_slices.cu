@@ -478,7 +478,7 @@ struct SplatSmem {
 template <int NX, int MB = -1>
 __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX, SplatCfg<NX>>())
     k_splat_row(Geo geo, Band b, const AtomRec* __restrict__ recs, const int* __restrict__ boffs, int A, int S,
-                int s0, int sb, int npair, int nbatch, float beta, float2* __restrict__ Bp) {
+                int s0, int sb, int npair, int two, int nbatch, float beta, float2* __restrict__ Bp) {
   constexpr int E = SplatCfg<NX>::E, T = SplatCfg<NX>::T, G = SplatCfg<NX>::G, NT = SplatCfg<NX>::THREADS;
   constexpr int PL = Tuned<K_SPLAT_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -495,7 +495,10 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
 
   const int bidx = batch_index();
   if (bidx >= nbatch) return;
-  const int pair = bidx % npair, fs = bidx / npair, f = fs / sb, s = s0 + fs % sb;
+  // two: the planes are pairs of slices (2i, 2i + 1) of the one species, the second as imaginary part;
+  // else slices, the odd slots of a species pair as imaginary part
+  const int pair = bidx % npair, fs = bidx / npair, f = fs / sb;
+  const int sa = two ? 2 * (s0 / 2 + fs % sb) : s0 + fs % sb, nhalf = two && sa + 1 < S ? 2 : 1;
   const int tid = threadIdx.x, g = tid / T, t = tid % T;
   const int ny = geo.ny, y0 = blockIdx.x * G;
   const AtomRec* R = recs + (size_t)f * A;
@@ -503,95 +506,99 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
   // footprints [iy0 + 1 - h, iy0 + h] meet rows [y0, y0 + G)), at most two contiguous ranges of
   // the row-sorted slice list (the window may wrap around y = 0)
   const int nyb = ny / SPREAD_YB;
-  const int* bo = boffs + ((size_t)f * S + s) * (nyb + 1);
   const int wlo = y0 - h, whi = y0 + G - 2 + h;
   const int b_lo = wlo >= 0 ? wlo / SPREAD_YB : -((-wlo + SPREAD_YB - 1) / SPREAD_YB), b_hi = whi / SPREAD_YB;
-  int s1, n1, s2 = 0, n2 = 0;
   const bool whole = b_hi - b_lo + 1 >= nyb;
-  if (whole) {
-    s1 = bo[0];
-    n1 = bo[nyb] - s1;
-  } else if (b_lo < 0) {
-    s1 = bo[b_lo + nyb];
-    n1 = bo[nyb] - s1;
-    s2 = bo[0];
-    n2 = bo[b_hi + 1] - s2;
-  } else if (b_hi >= nyb) {
-    s1 = bo[b_lo];
-    n1 = bo[nyb] - s1;
-    s2 = bo[0];
-    n2 = bo[b_hi - nyb + 1] - s2;
-  } else {
-    s1 = bo[b_lo];
-    n1 = bo[b_hi + 1] - s1;
-  }
-  const int M = n1 + n2;
 
 #pragma unroll
   for (int e = 0; e < E; ++e) acc[g * NX + t + T * e] = make_float2(0.f, 0.f);
 
-  for (int base = 0; base < M; base += NT) {
-    // 1. the batch's candidate records (atoms of other species pairs are marked and skipped)
-    const int j = base + tid;
-    if (j < M) {
-      const AtomRec r = R[j < n1 ? s1 + j : s2 + (j - n1)];
-      const int slot = r.jslot >> 24;
-      cfx[tid] = r.fx;
-      cfy[tid] = r.fy;
-      cx0[tid] = wrap3<NX>((r.ixy & 0xffff) + 1 - h + NX) | ((slot & 1) << 16);
-      const int iy = r.ixy >> 16;
-      ciy[tid] = (slot >> 1) == pair ? iy : -1;
-      int dy = iy - SPREAD_YB * b_lo;  // rows above the first candidate block
-      dy += dy < 0 ? ny : 0;
-      crow[tid] = dy - (dy >= ny ? ny : 0) + SPREAD_YB * b_lo - y0;
+  for (int half = 0; half < nhalf; ++half) {
+    const int* bo = boffs + ((size_t)f * S + sa + half) * (nyb + 1);
+    int s1, n1, s2 = 0, n2 = 0;
+    if (whole) {
+      s1 = bo[0];
+      n1 = bo[nyb] - s1;
+    } else if (b_lo < 0) {
+      s1 = bo[b_lo + nyb];
+      n1 = bo[nyb] - s1;
+      s2 = bo[0];
+      n2 = bo[b_hi + 1] - s2;
+    } else if (b_hi >= nyb) {
+      s1 = bo[b_lo];
+      n1 = bo[nyb] - s1;
+      s2 = bo[0];
+      n2 = bo[b_hi - nyb + 1] - s2;
+    } else {
+      s1 = bo[b_lo];
+      n1 = bo[b_hi + 1] - s1;
     }
-    __syncthreads();
-    const int total = M - base < NT ? M - base : NT;
-    // 2. kernel tables, one entry per thread: phx[c][d] (d < 2h) and phy[c][g]
-    const int per = W2 + G;
-    for (int i = tid; i < total * per; i += NT) {
-      const int c = i / per, k = i - c * per;
-      if (k < W2) {
-        phx[c * W2 + k] = es_kernel(((float)(k + 1 - h) - cfx[c]) / (float)h, beta);
-      } else {
-        const int gg = k - W2, cy = ciy[c];
-        int d = wrap3(y0 + gg - cy + ny, ny);
-        if (d > ny / 2) d -= ny;
-        phy[c * G + gg] = (cy >= 0 && d >= 1 - h && d <= h) ? es_kernel(((float)d - cfy[c]) / (float)h, beta)
-                                                           : 0.f;
+    const int M = n1 + n2;
+
+
+    for (int base = 0; base < M; base += NT) {
+      // 1. the batch's candidate records (atoms of other species pairs are marked and skipped)
+      const int j = base + tid;
+      if (j < M) {
+        const AtomRec r = R[j < n1 ? s1 + j : s2 + (j - n1)];
+        const int slot = r.jslot >> 24;
+        cfx[tid] = r.fx;
+        cfy[tid] = r.fy;
+        cx0[tid] = wrap3<NX>((r.ixy & 0xffff) + 1 - h + NX) | ((two ? half : slot & 1) << 16);
+        const int iy = r.ixy >> 16;
+        ciy[tid] = (slot >> 1) == pair ? iy : -1;
+        int dy = iy - SPREAD_YB * b_lo;  // rows above the first candidate block
+        dy += dy < 0 ? ny : 0;
+        crow[tid] = dy - (dy >= ny ? ny : 0) + SPREAD_YB * b_lo - y0;
       }
-    }
-    __syncthreads();
-    // 3. taps: thread (g, t) owns columns t + T e; a footprint of 2h columns starting at x0
-    //    meets them at the offsets congruent to t - x0 modulo T.  The candidates come in row order
-    //    (when they are not the whole slice), so those whose footprints hold this warp's rows are
-    //    one run of them; walking all of them took 512 points x
-    //    128 slices 117 us, this 99.
-    int c0 = 0, c1 = total;
-    if (!whole) {
-      const int lane = tid & 31, g0 = (tid - lane) / T, g1 = (tid - lane + 31) / T;  // rows of this warp
-      c1 = 0;
-      for (int c = 0; c < total; c += 32) {
-        const int r = c + lane < total ? crow[c + lane] : ny;
-        c0 += __popc(__ballot_sync(0xffffffffu, r < g0 - h));
-        c1 += __popc(__ballot_sync(0xffffffffu, r <= g1 - 1 + h));
+      __syncthreads();
+      const int total = M - base < NT ? M - base : NT;
+      // 2. kernel tables, one entry per thread: phx[c][d] (d < 2h) and phy[c][g]
+      const int per = W2 + G;
+      for (int i = tid; i < total * per; i += NT) {
+        const int c = i / per, k = i - c * per;
+        if (k < W2) {
+          phx[c * W2 + k] = es_kernel(((float)(k + 1 - h) - cfx[c]) / (float)h, beta);
+        } else {
+          const int gg = k - W2, cy = ciy[c];
+          int d = wrap3(y0 + gg - cy + ny, ny);
+          if (d > ny / 2) d -= ny;
+          phy[c * G + gg] = (cy >= 0 && d >= 1 - h && d <= h) ? es_kernel(((float)d - cfy[c]) / (float)h, beta)
+                                                             : 0.f;
+        }
       }
-    }
-    float* arow = reinterpret_cast<float*>(acc + g * NX);
-    float wy = c0 < c1 ? phy[c0 * G + g] : 0.f;
-    int xi = c0 < c1 ? cx0[c0] : 0;
-    for (int c = c0; c < c1; ++c) {
-      const float wyc = wy;
-      const int x0 = xi & 0xffff, im = xi >> 16;
-      if (c + 1 < c1) {
-        wy = phy[(c + 1) * G + g];
-        xi = cx0[c + 1];
+      __syncthreads();
+      // 3. taps: thread (g, t) owns columns t + T e; a footprint of 2h columns starting at x0
+      //    meets them at the offsets congruent to t - x0 modulo T.  The candidates come in row order
+      //    (when they are not the whole slice), so those whose footprints hold this warp's rows are
+      //    one run of them; walking all of them took 512 points x
+      //    128 slices 117 us, this 99.
+      int c0 = 0, c1 = total;
+      if (!whole) {
+        const int lane = tid & 31, g0 = (tid - lane) / T, g1 = (tid - lane + 31) / T;  // rows of this warp
+        c1 = 0;
+        for (int c = 0; c < total; c += 32) {
+          const int r = c + lane < total ? crow[c + lane] : ny;
+          c0 += __popc(__ballot_sync(0xffffffffu, r < g0 - h));
+          c1 += __popc(__ballot_sync(0xffffffffu, r <= g1 - 1 + h));
+        }
       }
-      if (wyc == 0.f) continue;
-      const int d = wrap3<NX>(x0 - t + NX);
-      for (int off = (T - d % T) % T; off < W2; off += T) arow[2 * wrap3<NX>(x0 + off) + im] += wyc * phx[c * W2 + off];
+      float* arow = reinterpret_cast<float*>(acc + g * NX);
+      float wy = c0 < c1 ? phy[c0 * G + g] : 0.f;
+      int xi = c0 < c1 ? cx0[c0] : 0;
+      for (int c = c0; c < c1; ++c) {
+        const float wyc = wy;
+        const int x0 = xi & 0xffff, im = xi >> 16;
+        if (c + 1 < c1) {
+          wy = phy[(c + 1) * G + g];
+          xi = cx0[c + 1];
+        }
+        if (wyc == 0.f) continue;
+        const int d = wrap3<NX>(x0 - t + NX);
+        for (int off = (T - d % T) % T; off < W2; off += T) arow[2 * wrap3<NX>(x0 + off) + im] += wyc * phx[c * W2 + off];
+      }
+      __syncthreads();
     }
-    __syncthreads();
   }
   float2 v[E];
 #pragma unroll
@@ -660,41 +667,71 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
 // sincosf brings a large-argument path that, unrolled over a thread's elements, overflowed the
 // instruction cache (no_instruction was the first stall): 512 points, 128 slices 134 -> 105 us; the
 // pass from V at 1024 points, 80 slices 552 -> 244 us.
-template <int NX, int MB = -1>
+// PAIR: a plane of Ap holds two slices of the one loaded species, V of the first in the real and of
+// the second in the imaginary part, so both take one inverse transform (and one spreading and one
+// column pass before it): three transforms per two rows instead of four here.  1152 points x 54 slices
+// x 20 frames: splat_row 4.10 -> 2.61 ms, col_pot 5.90 -> 3.05, this 7.08 -> 5.95.  A slice
+// without atoms is zero exactly, whatever its partner rounds to.
+template <int NX, bool PAIR, int MB = -1>
 __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT, NX, PotOutCfg<NX>>())
-    k_row_pot_out(Geo geo, Band b, const float2* __restrict__ Ap, int nbatch, int mode, float sigma,
+    k_row_pot_out(Geo geo, Band b, const float2* __restrict__ Ap, int nbatch, SlicePairs sp, int mode, float sigma,
                   float* __restrict__ V, float2* __restrict__ out) {
   constexpr int E = PotOutCfg<NX>::E, T = PotOutCfg<NX>::T, G = PotOutCfg<NX>::G;
   constexpr int PL = Tuned<K_ROW_POT_OUT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
-  const int fs = batch_index();
-  if (fs >= nbatch) return;
+  const int bi = batch_index();
+  if (bi >= nbatch) return;
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
   const RowIdx<NX, E> idx{g * row_smem_stride<NX, E>()};
   const auto sync = group_sync<T>(g);
   float2 v[E];
-  load_row<NX, MB>(v, Ap + ((size_t)fs * ny + y) * b.Wp, b, t);
+  load_row<NX, MB>(v, Ap + ((size_t)bi * ny + y) * b.Wp, b, t);
   fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
-  const size_t row = ((size_t)fs * ny + y) * NX;
-  if (mode == 0) {
-#pragma unroll
-    for (int e = 0; e < E; ++e) V[row + t + T * e] = v[e].x;
-    return;
+  // slices [s, s_end) of frame f come from this plane, s - s_first its part
+  int f = 0, s_first = 0, s = 0, s_end = 1;
+  if (PAIR) {
+    f = bi / sp.planes;
+    s_first = 2 * (sp.s0 / 2 + bi - f * sp.planes);
+    s = s_first < sp.s0 ? sp.s0 : s_first;
+    s_end = s_first + 2 < sp.s0 + sp.sb ? s_first + 2 : sp.s0 + sp.sb;
   }
+  float im[E];
 #pragma unroll
-  for (int e = 0; e < E; ++e) {
-    float sn, cs;
-    sincospif(sigma * v[e].x, &sn, &cs);
-    v[e] = make_float2(cs, sn);
-  }
-  if (mode == 2) {
+  for (int e = 0; e < E; ++e) im[e] = v[e].y;
+#pragma unroll 1
+  for (; s < s_end; ++s) {
+    float scale = 1.f;
+    if (PAIR) {
+      const int* bo = sp.boffs + ((size_t)f * sp.S + s) * (ny / SPREAD_YB + 1);
+      scale = bo[ny / SPREAD_YB] > bo[0] ? 1.f : 0.f;
+      if (s > s_first) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
-    return;
+        for (int e = 0; e < E; ++e) v[e].x = im[e];
+      }
+    }
+    const size_t plane = PAIR ? (size_t)f * sp.sb + (s - sp.s0) : (size_t)bi;
+    const size_t row = (plane * ny + y) * NX;
+    if (mode == 0) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) V[row + t + T * e] = PAIR ? scale * v[e].x : v[e].x;
+      continue;
+    }
+    const float sc = PAIR ? scale * sigma : sigma;
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      float sn, cs;
+      sincospif(sc * v[e].x, &sn, &cs);
+      v[e] = make_float2(cs, sn);
+    }
+    if (mode == 2) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
+      continue;
+    }
+    fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
+    store_row<NX, MB>(v, out + (plane * ny + y) * b.Wp, b, t);
   }
-  fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
-  store_row<NX, MB>(v, out + ((size_t)fs * ny + y) * b.Wp, b, t);
 }
 
 // ============================================================================================
@@ -1155,9 +1192,10 @@ constexpr int std_band_wp(int n) {
 
 template <int NX>
 static cudaError_t splat_row_n(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A,
-                               int S, int s0, int sb, int nfs, int npair, float beta, float2* Bp,
+                               int S, int s0, int sb, int nfs, int npair, int two, float beta, float2* Bp,
                                int static_band, cudaStream_t st) {
-  if (s0 < 0 || sb < 1 || s0 + sb > S || nfs % sb != 0) return cudaErrorInvalidValue;
+  if (s0 < 0 || sb < 1 || nfs % sb != 0 || (two ? npair != 1 || 2 * (s0 / 2 + sb - 1) >= S : s0 + sb > S))
+    return cudaErrorInvalidValue;
   const int smem = SplatSmem<NX>::BYTES;
   const int nb = nfs * npair;
   const dim3 grid = batch_grid(g.ny / SplatCfg<NX>::G, nb);
@@ -1166,22 +1204,22 @@ static cudaError_t splat_row_n(const Geo& g, const Band& b, const AtomRec* recs,
     if (std_band<NX>(b, static_band)) {
       cudaError_t e = prep(k_splat_row<NX, NX / 3>, smem);
       if (e != cudaSuccess) return e;
-      k_splat_row<NX, NX / 3><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb,
-                                                                          npair, nb, beta, Bp);
+      k_splat_row<NX, NX / 3><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb, npair,
+                                                                        two, nb, beta, Bp);
       return cudaGetLastError();
     }
   }
   cudaError_t e = prep(k_splat_row<NX>, smem);
   if (e != cudaSuccess) return e;
-  k_splat_row<NX><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb, npair, nb, beta,
-                                                             Bp);
+  k_splat_row<NX><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb,
+                                                             beta, Bp);
   return cudaGetLastError();
 }
 cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A, int S,
-                             int s0, int sb, int nfs, int npair, float beta, float2* Bp, int static_band,
+                             int s0, int sb, int nfs, int npair, int two, float beta, float2* Bp, int static_band,
                              cudaStream_t st) {
   if (g.ny % SPREAD_YB != 0) return cudaErrorInvalidValue;
-  TACAW_DISPATCH(g.nx, splat_row_n, g, b, recs, boffs, A, S, s0, sb, nfs, npair, beta, Bp, static_band, st);
+  TACAW_DISPATCH(g.nx, splat_row_n, g, b, recs, boffs, A, S, s0, sb, nfs, npair, two, beta, Bp, static_band, st);
 }
 
 template <int NY>
@@ -1217,23 +1255,29 @@ cudaError_t launch_col_pot(const Geo& g, const Band& b, const float2* Bp, const 
   TACAW_DISPATCH(g.ny, col_pot_n, g, b, Bp, mtab, npair, nfs, Ap, static_band, st);
 }
 
-template <int NX>
-static cudaError_t row_pot_out_n(const Geo& g, const Band& b, const float2* Ap, int nfs, int mode, float sigma,
-                                 float* V, float2* out, int static_band, cudaStream_t st) {
-  const dim3 grid = batch_grid(g.ny / PotOutCfg<NX>::G, nfs);
+template <int NX, bool PAIR>
+static cudaError_t row_pot_out_p(const Geo& g, const Band& b, const float2* Ap, int nb, const SlicePairs& sp, int mode,
+                                 float sigma, float* V, float2* out, int static_band, cudaStream_t st) {
+  using RC = PotOutCfg<NX>;
+  const dim3 grid = batch_grid(g.ny / RC::G, nb);
   if constexpr (std_band_built<NX>()) {
     if (std_band<NX>(b, static_band)) {
-      k_row_pot_out<NX, NX / 3><<<grid, PotOutCfg<NX>::THREADS, PotOutCfg<NX>::SMEM, st>>>(g, b, Ap, nfs, mode,
-                                                                                           sigma, V, out);
+      k_row_pot_out<NX, PAIR, NX / 3><<<grid, RC::THREADS, RC::SMEM, st>>>(g, b, Ap, nb, sp, mode, sigma, V, out);
       return cudaGetLastError();
     }
   }
-  k_row_pot_out<NX><<<grid, PotOutCfg<NX>::THREADS, PotOutCfg<NX>::SMEM, st>>>(g, b, Ap, nfs, mode, sigma, V, out);
+  k_row_pot_out<NX, PAIR><<<grid, RC::THREADS, RC::SMEM, st>>>(g, b, Ap, nb, sp, mode, sigma, V, out);
   return cudaGetLastError();
 }
-cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, int nfs, int mode, float sigma,
-                               float* V, float2* out, int static_band, cudaStream_t st) {
-  TACAW_DISPATCH(g.nx, row_pot_out_n, g, b, Ap, nfs, mode, sigma, V, out, static_band, st);
+template <int NX>
+static cudaError_t row_pot_out_n(const Geo& g, const Band& b, const float2* Ap, int nb, const SlicePairs& sp, int mode,
+                                 float sigma, float* V, float2* out, int static_band, cudaStream_t st) {
+  return sp.planes ? row_pot_out_p<NX, true>(g, b, Ap, nb, sp, mode, sigma, V, out, static_band, st)
+                   : row_pot_out_p<NX, false>(g, b, Ap, nb, sp, mode, sigma, V, out, static_band, st);
+}
+cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, int nb, const SlicePairs& sp, int mode,
+                               float sigma, float* V, float2* out, int static_band, cudaStream_t st) {
+  TACAW_DISPATCH(g.nx, row_pot_out_n, g, b, Ap, nb, sp, mode, sigma, V, out, static_band, st);
 }
 
 template <int NX>

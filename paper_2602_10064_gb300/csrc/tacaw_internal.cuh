@@ -179,16 +179,25 @@ cudaError_t launch_sort_rows(const AtomRec* recs, const int* offs, int64_t A, in
                              AtomRec* out, int* boffs, cudaStream_t st);
 // Spreading row pass of slices [s0, s0 + sb) of nfs / sb frames (batch = (frame, slice, pair)),
 // from the row-sorted records and their row-block offsets.
+// With `two` (one species loaded, npair 1) the planes are pairs of slices instead, (2i, 2i + 1) from
+// i = s0 / 2 on, sb of them per frame.
 cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A, int S,
-                             int s0, int sb, int nfs, int npair, float beta, float2* Bp, int static_band,
+                             int s0, int sb, int nfs, int npair, int two, float beta, float2* Bp, int static_band,
                              cudaStream_t st);
 cudaError_t launch_col_pot(const Geo& g, const Band& b, const float2* Bp, const float2* mtab, int npair, int nfs,
                            float2* Ap, int static_band, cudaStream_t st);
 // sigma_pi: the interaction parameter over pi.
 // mode 0: store V; mode 1: t = exp(i sigma V), band-limit pass input (FFT_x, compact);
 // mode 2: t = exp(i sigma V) stored directly (no transmission band limit).
-cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, int nfs, int mode, float sigma,
-                               float* V, float2* out, int static_band, cudaStream_t st);
+// Ap: nb planes.  sp.planes = 0: a plane per slice, written to the same plane of the output.  Else
+// sp.planes planes per frame, each a pair of slices (2i, 2i + 1), i from s0 / 2 on; the slices
+// [s0, s0 + sb) are written, sb planes per frame; boffs (of the first frame) tells empty slices.
+struct SlicePairs {
+  int planes, S, s0, sb;
+  const int* boffs;
+};
+cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, int nb, const SlicePairs& sp, int mode,
+                               float sigma, float* V, float2* out, int static_band, cudaStream_t st);
 cudaError_t launch_row_vt(const Geo& g, const Band& b, const float* V, int nfs, int bandlimit, float sigma,
                           float2* out, cudaStream_t st);
 cudaError_t launch_col_t(const Geo& g, const Band& b, const float2* Bt, int nfs, float scale, float2* At,
