@@ -268,6 +268,7 @@ __global__ void __launch_bounds__(256) k_slice_index(const float* __restrict__ p
 __global__ void __launch_bounds__(256) k_atoms(const float* __restrict__ pos, int A, int64_t nf, BinGeom g,
                                                const int8_t* __restrict__ slot_of_atom, AtomRec* __restrict__ rec,
                                                uint8_t* __restrict__ key) {
+  grid_dependency_wait();
   const int j = blockIdx.x * 256 + threadIdx.x;
   if (j >= A || batch_index() >= nf) return;
   const size_t at = (size_t)batch_index() * A + j;
@@ -285,6 +286,7 @@ __global__ void __launch_bounds__(256) k_atoms(const float* __restrict__ pos, in
 __global__ void __launch_bounds__(BIN_THREADS) k_bin(const AtomRec* __restrict__ rec, const uint8_t* __restrict__ key,
                                                       int A, int S, AtomRec* __restrict__ recs,
                                                       int* __restrict__ offs) {
+  grid_dependency_wait();
   __shared__ int counts[BIN_MAX_S];
   __shared__ int cursor[BIN_MAX_S];
   __shared__ int wcount[BIN_THREADS / 32][BIN_MAX_S];
@@ -331,6 +333,7 @@ __global__ void __launch_bounds__(BIN_THREADS) k_bin(const AtomRec* __restrict__
 
 __global__ void k_map_slots(const int32_t* __restrict__ Z, int64_t A, const int8_t* __restrict__ lut,
                             int8_t* __restrict__ slot, int* __restrict__ status) {
+  grid_dependency_wait();
   for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < A; j += (int64_t)gridDim.x * blockDim.x) {
     const int z = Z[j];
     int s = (z >= 0 && z < 256) ? lut[z] : -1;
@@ -346,8 +349,7 @@ cudaError_t launch_map_slots(const int32_t* Z, int64_t A, const int8_t* lut, int
                              cudaStream_t st) {
   if (A <= 0) return cudaSuccess;
   const int64_t blocks = (A + 255) / 256;
-  k_map_slots<<<(unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st>>>(Z, A, lut, slot, status);
-  return cudaGetLastError();
+  return launch_after(k_map_slots, (unsigned)(blocks < 1024 ? blocks : 1024), 256, 0, st, Z, A, lut, slot, status);
 }
 
 // One warp per (frame, slice): stable counting sort of the slice's atom records by the grid
@@ -358,6 +360,7 @@ constexpr int SORT_WARPS = 8;
 __global__ void __launch_bounds__(SORT_WARPS * 32)
     k_sort_rows(const AtomRec* __restrict__ recs, const int* __restrict__ offs, int A, int S, int nseg, int ny,
                 AtomRec* __restrict__ out, int* __restrict__ boffs) {
+  grid_dependency_wait();
   extern __shared__ int cnt_all[];  // [SORT_WARPS][ny]
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int seg = blockIdx.x * SORT_WARPS + warp;
@@ -423,9 +426,7 @@ cudaError_t launch_sort_rows(const AtomRec* recs, const int* offs, int64_t A, in
     const cudaError_t e = cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  k_sort_rows<<<(unsigned)((nseg + SORT_WARPS - 1) / SORT_WARPS), SORT_WARPS * 32, smem, st>>>(
-      recs, offs, (int)A, S, (int)nseg, ny, out, boffs);
-  return cudaGetLastError();
+  return launch_after(k_sort_rows, (unsigned)((nseg + SORT_WARPS - 1) / SORT_WARPS), SORT_WARPS * 32, smem, st,  recs, offs, (int)A, S, (int)nseg, ny, out, boffs);
 }
 
 cudaError_t launch_slice_index(const float* pos, int64_t n, const BinGeom& g, int* slice_out, cudaStream_t st) {
@@ -437,11 +438,10 @@ cudaError_t launch_slice_index(const float* pos, int64_t n, const BinGeom& g, in
 cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, const BinGeom& g, const int8_t* slot_of_atom,
                        AtomRec* rec, uint8_t* key, AtomRec* recs, int* offs, cudaStream_t st) {
   if (g.S > BIN_MAX_S || nf <= 0) return cudaErrorInvalidValue;
-  if (A > 0) k_atoms<<<batch_grid((int)((A + 255) / 256), nf), 256, 0, st>>>(pos, (int)A, nf, g, slot_of_atom, rec, key);
-  cudaError_t e = cudaGetLastError();
+  cudaError_t e = cudaSuccess;
+  if (A > 0) e = launch_after(k_atoms, batch_grid((int)((A + 255) / 256), nf), 256, 0, st, pos, (int)A, nf, g, slot_of_atom, rec, key);
   if (e != cudaSuccess) return e;
-  k_bin<<<(unsigned)nf, BIN_THREADS, 0, st>>>(rec, key, (int)A, g.S, recs, offs);
-  return cudaGetLastError();
+  return launch_after(k_bin, (unsigned)nf, BIN_THREADS, 0, st, rec, key, (int)A, g.S, recs, offs);
 }
 
 // ============================================================================================
@@ -479,6 +479,7 @@ template <int NX, int MB = -1>
 __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX, SplatCfg<NX>>())
     k_splat_row(Geo geo, Band b, const AtomRec* __restrict__ recs, const int* __restrict__ boffs, int A, int S,
                 int s0, int sb, int npair, int two, int nbatch, float beta, float2* __restrict__ Bp) {
+  grid_dependency_wait();
   constexpr int E = SplatCfg<NX>::E, T = SplatCfg<NX>::T, G = SplatCfg<NX>::G, NT = SplatCfg<NX>::THREADS;
   constexpr int PL = Tuned<K_SPLAT_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -614,6 +615,7 @@ template <int NY, bool ONE, int WPC = -1>
 __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY, ColPotCfg<NY>>())
     k_col_pot(Geo geo, Band b, const float2* __restrict__ Bp, const float2* __restrict__ mtab, int npair, int nbatch,
               float2* __restrict__ Ap) {
+  grid_dependency_wait();
   using CC = ColPotCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
   constexpr int PL = Tuned<K_COL_POT, NY>::PLAN;
@@ -676,6 +678,7 @@ template <int NX, bool PAIR, int MB = -1>
 __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT, NX, PotOutCfg<NX>>())
     k_row_pot_out(Geo geo, Band b, const float2* __restrict__ Ap, int nbatch, SlicePairs sp, int mode, float sigma,
                   float* __restrict__ V, float2* __restrict__ out) {
+  grid_dependency_wait();
   constexpr int E = PotOutCfg<NX>::E, T = PotOutCfg<NX>::T, G = PotOutCfg<NX>::G;
   constexpr int PL = Tuned<K_ROW_POT_OUT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -741,6 +744,7 @@ template <int NX>
 __global__ void __launch_bounds__(RowVtCfg<NX>::THREADS, minb_of<K_ROW_VT, NX, RowVtCfg<NX>>())
     k_row_vt(Geo geo, Band b, const float* __restrict__ V, int nbatch, int bandlimit, float sigma,
              float2* __restrict__ out) {
+  grid_dependency_wait();
   constexpr int E = RowVtCfg<NX>::E, T = RowVtCfg<NX>::T, G = RowVtCfg<NX>::G;
   constexpr int PL = Tuned<K_ROW_VT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -770,6 +774,7 @@ __global__ void __launch_bounds__(RowVtCfg<NX>::THREADS, minb_of<K_ROW_VT, NX, R
 template <int NY, int WPC = -1>
 __global__ void __launch_bounds__(ColTCfg<NY>::THREADS, minb_of<K_COL_T, NY, ColTCfg<NY>>())
     k_col_t(Geo geo, Band b, const float2* __restrict__ Bt, int nbatch, float scale, float2* __restrict__ At) {
+  grid_dependency_wait();
   using CC = ColTCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
   constexpr int PL = Tuned<K_COL_T, NY>::PLAN;
@@ -803,6 +808,7 @@ __global__ void __launch_bounds__(ColTCfg<NY>::THREADS, minb_of<K_COL_T, NY, Col
 template <int NX>
 __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, NX, RowToutCfg<NX>>())
     k_row_tout(Geo geo, Band b, const float2* __restrict__ At, int nbatch, float2* __restrict__ tout) {
+  grid_dependency_wait();
   constexpr int E = RowToutCfg<NX>::E, T = RowToutCfg<NX>::T, G = RowToutCfg<NX>::G;
   constexpr int PL = Tuned<K_ROW_TOUT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -830,6 +836,7 @@ __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, N
 __global__ void __launch_bounds__(256) k_probe_tables(ProbeTables q, const double* __restrict__ xy,
                                                       const int* __restrict__ nb, float2* __restrict__ ex,
                                                       float2* __restrict__ ey, float2* __restrict__ chi) {
+  grid_dependency_wait();
   const int64_t nex = (int64_t)q.P * q.Wp, ney = (int64_t)q.P * q.ny, nchi = chi ? (int64_t)q.ny * q.Wp : 0;
   for (int64_t i = blockIdx.x * (int64_t)256 + threadIdx.x; i < nex + ney + nchi; i += (int64_t)gridDim.x * 256) {
     double s, c;
@@ -866,14 +873,14 @@ __global__ void __launch_bounds__(256) k_probe_tables(ProbeTables q, const doubl
 cudaError_t launch_probe_tables(const ProbeTables& q, const double* xy, const int* nb, float2* ex, float2* ey,
                                 float2* chi, cudaStream_t st) {
   const int64_t n = (int64_t)q.P * (q.Wp + q.ny) + (chi ? (int64_t)q.ny * q.Wp : 0);
-  k_probe_tables<<<(unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st>>>(q, xy, nb, ex, ey, chi);
-  return cudaGetLastError();
+  return launch_after(k_probe_tables, (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st, q, xy, nb, ex, ey, chi);
 }
 
 template <int NY>
 __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL, NY, ProbeColCfg<NY>>())
     k_probe_col(Geo geo, Band ap, const float2* __restrict__ ex, const float2* __restrict__ ey,
                 const float2* __restrict__ chi, int P, float amp, float2* __restrict__ Bpr) {
+  grid_dependency_wait();
   using CC = ProbeColCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
   constexpr int PL = Tuned<K_PROBE_COL, NY>::PLAN;
@@ -900,6 +907,7 @@ __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL,
 template <int NX>
 __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW, NX, ProbeRowCfg<NX>>())
     k_probe_row(Geo geo, Band ap, const float2* __restrict__ Bpr, int P, float scale, float2* __restrict__ psi0) {
+  grid_dependency_wait();
   constexpr int E = ProbeRowCfg<NX>::E, T = ProbeRowCfg<NX>::T, G = ProbeRowCfg<NX>::G;
   constexpr int PL = Tuned<K_PROBE_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -949,6 +957,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
     k_slice_row(Geo geo, Band b, const float2* __restrict__ Apsi, const float2* __restrict__ psi0,
                 const float2* __restrict__ ttab, int S, int s, int P, int ppb, int nfc, int nbatch, float plane_amp,
                 float2* __restrict__ Bpsi) {
+  grid_dependency_wait();
   using RC = SliceRowCfg<NX, TF>;
   constexpr int E = RC::E, T = RC::T, G = RC::G;
   constexpr int PL = Tuned<slice_row_id<TF>(), NX>::PLAN;
@@ -1036,6 +1045,7 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
     k_slice_col(Geo geo, Band b, const float2* __restrict__ Bpsi, const float2* __restrict__ px,
                 const float2* __restrict__ py, float scale, int wpb, int nfc, int nwaves, int64_t F_total, int64_t f0,
                 const int2* __restrict__ disc, int64_t nsel, float2* __restrict__ Apsi, float2* __restrict__ psi_k) {
+  grid_dependency_wait();
   using CC = SliceColCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
   constexpr int PL = Tuned<K_SLICE_COL, NY>::PLAN;
@@ -1204,16 +1214,12 @@ static cudaError_t splat_row_n(const Geo& g, const Band& b, const AtomRec* recs,
     if (std_band<NX>(b, static_band)) {
       cudaError_t e = prep(k_splat_row<NX, NX / 3>, smem);
       if (e != cudaSuccess) return e;
-      k_splat_row<NX, NX / 3><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb, npair,
-                                                                        two, nb, beta, Bp);
-      return cudaGetLastError();
+      return launch_after(k_splat_row<NX, NX / 3>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb, beta, Bp);
     }
   }
   cudaError_t e = prep(k_splat_row<NX>, smem);
   if (e != cudaSuccess) return e;
-  k_splat_row<NX><<<grid, SplatCfg<NX>::THREADS, smem, st>>>(g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb,
-                                                             beta, Bp);
-  return cudaGetLastError();
+  return launch_after(k_splat_row<NX>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb, beta, Bp);
 }
 cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A, int S,
                              int s0, int sb, int nfs, int npair, int two, float beta, float2* Bp, int static_band,
@@ -1233,20 +1239,20 @@ static cudaError_t col_pot_n(const Geo& g, const Band& b, const float2* Bp, cons
     if (g.nx == NY && b.Wp == WP && std_band<NY>(b, static_band)) {
       if (npair == 1) {
         if ((e = prep(k_col_pot<NY, true, WP>, CC::SMEM)) != cudaSuccess) return e;
-        k_col_pot<NY, true, WP><<<grid, CC::THREADS, CC::SMEM, st>>>(g, b, Bp, mtab, npair, nfs, Ap);
+        return launch_after(k_col_pot<NY, true, WP>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
       } else {
         if ((e = prep(k_col_pot<NY, false, WP>, CC::SMEM)) != cudaSuccess) return e;
-        k_col_pot<NY, false, WP><<<grid, CC::THREADS, CC::SMEM, st>>>(g, b, Bp, mtab, npair, nfs, Ap);
+        return launch_after(k_col_pot<NY, false, WP>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
       }
       return cudaGetLastError();
     }
   }
   if (npair == 1) {
     if ((e = prep(k_col_pot<NY, true>, CC::SMEM)) != cudaSuccess) return e;
-    k_col_pot<NY, true><<<grid, CC::THREADS, CC::SMEM, st>>>(g, b, Bp, mtab, npair, nfs, Ap);
+    return launch_after(k_col_pot<NY, true>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
   } else {
     if ((e = prep(k_col_pot<NY, false>, CC::SMEM)) != cudaSuccess) return e;
-    k_col_pot<NY, false><<<grid, CC::THREADS, CC::SMEM, st>>>(g, b, Bp, mtab, npair, nfs, Ap);
+    return launch_after(k_col_pot<NY, false>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
   }
   return cudaGetLastError();
 }
@@ -1262,12 +1268,10 @@ static cudaError_t row_pot_out_p(const Geo& g, const Band& b, const float2* Ap, 
   const dim3 grid = batch_grid(g.ny / RC::G, nb);
   if constexpr (std_band_built<NX>()) {
     if (std_band<NX>(b, static_band)) {
-      k_row_pot_out<NX, PAIR, NX / 3><<<grid, RC::THREADS, RC::SMEM, st>>>(g, b, Ap, nb, sp, mode, sigma, V, out);
-      return cudaGetLastError();
+      return launch_after(k_row_pot_out<NX, PAIR, NX / 3>, grid, RC::THREADS, RC::SMEM, st, g, b, Ap, nb, sp, mode, sigma, V, out);
     }
   }
-  k_row_pot_out<NX, PAIR><<<grid, RC::THREADS, RC::SMEM, st>>>(g, b, Ap, nb, sp, mode, sigma, V, out);
-  return cudaGetLastError();
+  return launch_after(k_row_pot_out<NX, PAIR>, grid, RC::THREADS, RC::SMEM, st, g, b, Ap, nb, sp, mode, sigma, V, out);
 }
 template <int NX>
 static cudaError_t row_pot_out_n(const Geo& g, const Band& b, const float2* Ap, int nb, const SlicePairs& sp, int mode,
@@ -1283,9 +1287,7 @@ cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, in
 template <int NX>
 static cudaError_t row_vt_n(const Geo& g, const Band& b, const float* V, int nfs, int bl, float sigma, float2* out,
                             cudaStream_t st) {
-  k_row_vt<NX><<<batch_grid(g.ny / RowVtCfg<NX>::G, nfs), RowVtCfg<NX>::THREADS, RowVtCfg<NX>::SMEM, st>>>(
-      g, b, V, nfs, bl, sigma, out);
-  return cudaGetLastError();
+  return launch_after(k_row_vt<NX>, batch_grid(g.ny / RowVtCfg<NX>::G, nfs), RowVtCfg<NX>::THREADS, RowVtCfg<NX>::SMEM, st,  g, b, V, nfs, bl, sigma, out);
 }
 cudaError_t launch_row_vt(const Geo& g, const Band& b, const float* V, int nfs, int bandlimit, float sigma,
                           float2* out, cudaStream_t st) {
@@ -1301,15 +1303,12 @@ static cudaError_t col_t_n(const Geo& g, const Band& b, const float2* Bt, int nf
     if (g.nx == NY && b.Wp == WP && std_band<NY>(b, static_band)) {
       const cudaError_t e = prep(k_col_t<NY, WP>, CC::SMEM);
       if (e != cudaSuccess) return e;
-      k_col_t<NY, WP><<<batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st>>>(g, b, Bt, nfs, scale, At);
-      return cudaGetLastError();
+      return launch_after(k_col_t<NY, WP>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt, nfs, scale, At);
     }
   }
   const cudaError_t e = prep(k_col_t<NY>, CC::SMEM);
   if (e != cudaSuccess) return e;
-  k_col_t<NY><<<batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st>>>(g, b, Bt, nfs,
-                                                                                                   scale, At);
-  return cudaGetLastError();
+  return launch_after(k_col_t<NY>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt, nfs, scale, At);
 }
 cudaError_t launch_col_t(const Geo& g, const Band& b, const float2* Bt, int nfs, float scale, float2* At,
                          int static_band, cudaStream_t st) {
@@ -1319,8 +1318,7 @@ cudaError_t launch_col_t(const Geo& g, const Band& b, const float2* Bt, int nfs,
 template <int NX>
 static cudaError_t row_tout_n(const Geo& g, const Band& b, const float2* At, int nfs, float2* t, cudaStream_t st) {
   using RC = RowToutCfg<NX>;
-  k_row_tout<NX><<<batch_grid(g.ny / RC::G, nfs), RC::THREADS, RC::SMEM, st>>>(g, b, At, nfs, t);
-  return cudaGetLastError();
+  return launch_after(k_row_tout<NX>, batch_grid(g.ny / RC::G, nfs), RC::THREADS, RC::SMEM, st, g, b, At, nfs, t);
 }
 cudaError_t launch_row_tout(const Geo& g, const Band& b, const float2* At, int nfs, float2* t, cudaStream_t st) {
   TACAW_DISPATCH(g.nx, row_tout_n, g, b, At, nfs, t, st);
@@ -1332,9 +1330,7 @@ static cudaError_t probe_col_n(const Geo& g, const Band& ap, const float2* ex, c
   using CC = ProbeColCfg<NY>;
   const cudaError_t e = prep(k_probe_col<NY>, CC::SMEM);
   if (e != cudaSuccess) return e;
-  k_probe_col<NY><<<batch_grid(col_blocks(ap, CC::C), P), CC::THREADS, CC::SMEM, st>>>(
-      g, ap, ex, ey, chi, P, amp, Bpr);
-  return cudaGetLastError();
+  return launch_after(k_probe_col<NY>, batch_grid(col_blocks(ap, CC::C), P), CC::THREADS, CC::SMEM, st,  g, ap, ex, ey, chi, P, amp, Bpr);
 }
 cudaError_t launch_probe_col(const Geo& g, const Band& ap, const float2* ex, const float2* ey, const float2* chi,
                              int P, float amp, float2* Bpr, cudaStream_t st) {
@@ -1345,8 +1341,7 @@ template <int NX>
 static cudaError_t probe_row_n(const Geo& g, const Band& ap, const float2* Bpr, int P, float scale, float2* psi0,
                                cudaStream_t st) {
   using RC = ProbeRowCfg<NX>;
-  k_probe_row<NX><<<batch_grid(g.ny / RC::G, P), RC::THREADS, RC::SMEM, st>>>(g, ap, Bpr, P, scale, psi0);
-  return cudaGetLastError();
+  return launch_after(k_probe_row<NX>, batch_grid(g.ny / RC::G, P), RC::THREADS, RC::SMEM, st, g, ap, Bpr, P, scale, psi0);
 }
 cudaError_t launch_probe_row(const Geo& g, const Band& ap, const float2* Bpr, int P, float scale, float2* psi0,
                              cudaStream_t st) {
@@ -1369,8 +1364,8 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
     constexpr int SM = SliceRowSmem<NX, TFU>::BYTES, TH = SliceRowCfg<NX, TFU>::THREADS;                          \
     cudaError_t e_ = prep(k_slice_row<NX, F, PL, TFU>, SM);                                                       \
     if (e_ != cudaSuccess) return e_;                                                                             \
-    k_slice_row<NX, F, PL, TFU><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch, plane_amp,      \
-                                                       Bpsi);                                                     \
+    return launch_after(k_slice_row<NX, F, PL, TFU>, grid, TH, SM, st, g, b, Apsi, psi0, t, S, s, P, ppb, nfc,     \
+                        nbatch, plane_amp, Bpsi);                                                                 \
   } while (0)
   // the later slices (all but one of S) with the standard band fixed at compile time
   constexpr int MB3 = NX / 3;
@@ -1381,8 +1376,8 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
     constexpr int SM = SliceRowSmem<NX, TFU>::BYTES, TH = SliceRowCfg<NX, TFU>::THREADS;                          \
     cudaError_t e_ = prep(k_slice_row<NX, false, false, TFU, MB3>, SM);                                           \
     if (e_ != cudaSuccess) return e_;                                                                             \
-    k_slice_row<NX, false, false, TFU, MB3><<<grid, TH, SM, st>>>(g, b, Apsi, psi0, t, S, s, P, ppb, nfc, nbatch,  \
-                                                                  plane_amp, Bpsi);                               \
+    return launch_after(k_slice_row<NX, false, false, TFU, MB3>, grid, TH, SM, st, g, b, Apsi, psi0, t, S, s, P,    \
+                        ppb, nfc, nbatch, plane_amp, Bpsi);                                                       \
   } while (0)
   if (tfused) {
     if (first && plane) TACAW_SLICE_ROW(true, true, true);
@@ -1429,9 +1424,8 @@ static cudaError_t slice_col_n(const Geo& g, const Band& b, int last, const floa
     constexpr int SM = CC::SMEM + ((LOOP) ? NY * CC::C * (int)sizeof(float2) : 0);                                      \
     cudaError_t e_ = prep(k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>, SM);                                   \
     if (e_ != cudaSuccess) return e_;                                                                                 \
-    k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>                                                               \
-        <<<grid, TH, SM, st>>>(g, b, Bpsi, px, py, scale, wpb, nfc, nw, F_total, f0, disc, nsel, Apsi, psi_k);        \
-    return cudaGetLastError();                                                                                        \
+    return launch_after(k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>, grid, TH, SM, st, g, b, Bpsi, px, py,     \
+                        scale, wpb, nfc, nw, F_total, f0, disc, nsel, Apsi, psi_k);                                   \
   } while (0)
   if (last) TACAW_SLICE_COL(true, false);
   // the later slices of a square grid with the standard band: row stride fixed at compile time

@@ -149,6 +149,7 @@ cudaError_t launch_dft_fp32(const float2* r, const float2* twF, int64_t P, int64
 constexpr int DP_BINS = 32, DP_GROUPS = 8;
 __global__ void __launch_bounds__(DP_BINS * DP_GROUPS)
     k_detector_parts(const double* __restrict__ part, int64_t F, int64_t nparts, float* __restrict__ SI) {
+  grid_dependency_wait();
   __shared__ double red[DP_GROUPS][DP_BINS];
   const int b = threadIdx.x % DP_BINS, g = threadIdx.x / DP_BINS;
   const int64_t m = blockIdx.x * (int64_t)DP_BINS + b, p = blockIdx.y;
@@ -166,9 +167,7 @@ __global__ void __launch_bounds__(DP_BINS * DP_GROUPS)
 cudaError_t launch_detector_parts(const double* part, int64_t P, int64_t F, int64_t nparts, float* SI,
                                   cudaStream_t st) {
   if (P > 65535) return cudaErrorInvalidValue;
-  k_detector_parts<<<dim3((unsigned)((F + DP_BINS - 1) / DP_BINS), (unsigned)P), DP_BINS * DP_GROUPS, 0, st>>>(
-      part, F, nparts, SI);
-  return cudaGetLastError();
+  return launch_after(k_detector_parts, dim3((unsigned)((F + DP_BINS - 1) / DP_BINS), (unsigned)P), DP_BINS * DP_GROUPS, 0, st,  part, F, nparts, SI);
 }
 
 // SI[p][m] = sum_j S[p][m][q_j], FP64 accumulation with a fixed reduction tree.

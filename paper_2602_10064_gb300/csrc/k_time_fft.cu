@@ -66,6 +66,7 @@ constexpr int TIME_DET_TILES = 8;
 
 template <int N, int OUT, bool BLUE>
 __global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_fft(const TimeArgs a) {
+  grid_dependency_wait();
   using TC = TimeCfg<N>;
   constexpr int E = TC::E, T = TC::T, C = TC::C, WARPS = TC::THREADS / 32;
   extern __shared__ __align__(16) unsigned char smraw[];
@@ -217,8 +218,7 @@ cudaError_t launch_n(const TimeArgs& a, cudaStream_t st) {
     const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, TC::SMEM);
     if (e != cudaSuccess) return e;
   }
-  k<<<dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), TC::THREADS, TC::SMEM, st>>>(a);
-  return cudaGetLastError();
+  return launch_after(k, dim3((unsigned)gx, (unsigned)gy, (unsigned)gz), TC::THREADS, TC::SMEM, st, a);
 }
 
 template <int N>

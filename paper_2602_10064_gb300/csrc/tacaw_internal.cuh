@@ -137,6 +137,35 @@ __device__ __forceinline__ int band_x_col(const Band& b, int nx, int x) {
   return x <= b.mb ? x : (x >= nx - b.mb ? x - nx + b.W : -1);
 }
 
+// Programmatic dependent launch: a kernel launched by launch_after may start once every block of the
+// kernel before it on the stream has started, and each of its threads waits here, before it touches
+// memory, until that kernel has completed and its writes are visible.  It hides the launch and the
+// ramp-up of the next kernel behind the last blocks of this one: a run is a chain of 25 to a thousand
+// launches.  Only for short kernels, of at most kDependentThreads threads (five fillings of the SMs
+// at 512 threads each): 128^2 x 64 frames 230 -> 185 us, 37 probes at 384^2 989 -> 884 us, a 192 x 96
+// scan 981 -> 903 us; with the long ones too, a 256^2 scan went from 93 to 107 ms and a 512^2 plane
+// wave from 23.2 to 27.1 ms.
+constexpr long long kDependentThreads = 5LL * 512 * 152;
+__device__ __forceinline__ void grid_dependency_wait() {
+  asm volatile("griddepcontrol.launch_dependents;");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <class... P, class... A>
+inline cudaError_t launch_after(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st,
+                                A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cfg.attrs = &at;
+  cfg.numAttrs = (long long)grid.x * grid.y * grid.z * threads <= kDependentThreads ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // ---- host launchers (k_slices.cu) ---------------------------------------------------------
 // Spreading kernel exp(beta (sqrt(1 - z^2) - 1)) over z = d / SPREAD_HALF: 2 SPREAD_HALF grid points.
 constexpr int SPREAD_HALF = 6;
