@@ -29,19 +29,48 @@
 
 namespace tacaw {
 
-// Elements per thread and columns per CTA of each length: 8 columns are 64-byte lines of the stack,
-// 16 or 32 whole lines; more columns of the long transforms would leave one CTA per SM.
-template <int N>
-struct TimeCfg {
-  static constexpr int E = !fft_pow2(N) ? 24 : N <= 64 ? 8 : N >= 2048 ? 32 : 16;
-  static constexpr int T = N / E;
-  static constexpr int C = N <= 128 ? 32 : N <= 512 ? 16 : N <= 2048 ? 8 : 4;
-  static constexpr int THREADS = T * C;
-  static constexpr int SMEM = N * C * (int)sizeof(float2);
-  static constexpr int MINB = E >= 24 ? 1 : (512 / THREADS < 1 ? 1 : 512 / THREADS);
-};
-
 enum TimeOut { TIME_S, TIME_DETECTOR, TIME_TILDE };
+
+// Shape of a kernel: elements per thread, columns per CTA, CTAs per SM, and whether a thread loads its
+// next column while it transforms this one.  Per length the fastest of 4 to 14 shapes on one GB300
+// (ps per element of the stack; one shape for all uses -> these): 256 points S 3.21 -> 2.95, image
+// 3.05 -> 2.85, chirp-z 7.64 -> 7.08; 512: S 4.99 -> 3.39, image 4.88 -> 3.14, chirp-z 11.4 -> 8.0;
+// 1024: S 7.02 -> 4.95, image 5.41 -> 4.42, chirp-z 13.0 -> 11.2; 2048: S 7.91 -> 7.54, image 7.43 ->
+// 5.87, chirp-z 19.8 -> 14.9; 4096: chirp-z 27.7 -> 16.9.  16 columns are whole 128-byte lines of the
+// stack; more columns of the long transforms would leave one CTA per SM.
+struct TimeShape {
+  int e, c, minb;
+  bool prefetch;
+};
+constexpr TimeShape time_shape(int n, int out, bool chirp) {
+  switch (n) {
+    case 32: return {8, 32, 4, !chirp};
+    case 64: return {8, 32, 2, !chirp};
+    case 96: return {24, 32, 2, false};
+    case 128: return {16, 32, 2, !chirp};
+    case 192: return {24, 16, 2, false};
+    case 256: return chirp ? TimeShape{16, 8, 4, false} : TimeShape{16, 16, out == TIME_DETECTOR ? 3 : 2, true};
+    case 384: return {24, 16, 1, false};
+    case 512: return chirp || out == TIME_DETECTOR ? TimeShape{32, 8, 3, false} : TimeShape{32, 16, 1, true};
+    case 768: return {24, 8, 1, false};
+    case 1024: return {32, 8, !chirp && out == TIME_DETECTOR ? 2 : 1, !chirp};
+    case 1152: return {24, 8, 1, false};
+    case 2048:
+      return chirp || out == TIME_DETECTOR ? TimeShape{32, 4, 1, false}
+             : out == TIME_S               ? TimeShape{16, 4, 1, true}
+                                           : TimeShape{32, 8, 1, false};
+    default: return {32, 2, 1, false};
+  }
+}
+template <int N, int OUT, bool BLUE>
+struct TimeCfg {
+  static constexpr TimeShape SHAPE = time_shape(N, OUT, BLUE);
+  static constexpr int E = SHAPE.e, T = N / E, C = SHAPE.c, THREADS = T * C, MINB = SHAPE.minb;
+  static constexpr int SH = E == 32 ? 5 : 0;
+  static constexpr int SMEM = (N + (SH ? N >> SH : 0)) * C * (int)sizeof(float2);
+  // the spectrum image keeps its running sums in those registers
+  static constexpr bool PREFETCH = SHAPE.prefetch && OUT != TIME_DETECTOR;
+};
 
 struct TimeArgs {
   const float2* psi;  // [P][nf][in_nq]
@@ -58,6 +87,7 @@ struct TimeArgs {
   const float2* tw;     // FFT pass tables
   const float2* chirp;  // Bluestein: exp(-i pi n^2 / F), n < F
   const float2* bhat;   // Bluestein: spectrum of the conjugate chirp over M
+  int tpc;              // column tiles per CTA
 };
 
 // Column tiles one CTA of the spectrum image adds up before it stores its partial sums.  Fixed, so
@@ -65,16 +95,16 @@ struct TimeArgs {
 constexpr int TIME_DET_TILES = 8;
 
 template <int N, int OUT, bool BLUE>
-__global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_fft(const TimeArgs a) {
+__global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT, BLUE>::MINB) k_time_fft(const TimeArgs a) {
   grid_dependency_wait();
-  using TC = TimeCfg<N>;
+  using TC = TimeCfg<N, OUT, BLUE>;
   constexpr int E = TC::E, T = TC::T, C = TC::C, WARPS = TC::THREADS / 32;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int64_t p = blockIdx.y + (int64_t)gridDim.y * blockIdx.z;
   if (p >= a.P) return;
   const int c = threadIdx.x % C, t = threadIdx.x / C;
-  const ColIdx<C, 0> idx{c};
+  const ColIdx<C, TC::SH> idx{c};
   const BlockSync sync;
   const int F = (int)a.F;
   const int64_t ntiles = (a.nsel + C - 1) / C;
@@ -83,32 +113,41 @@ __global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_
 #pragma unroll
     for (int e = 0; e < E; ++e) hi[e] = lo[e] = 0.f;
   }
-  const int64_t tile0 = OUT == TIME_DETECTOR ? (int64_t)blockIdx.x * TIME_DET_TILES : blockIdx.x;
-  const int64_t tile1 = OUT == TIME_DETECTOR ? (tile0 + TIME_DET_TILES < ntiles ? tile0 + TIME_DET_TILES : ntiles)
-                                             : tile0 + 1;
-  for (int64_t tile = tile0; tile < tile1; ++tile) {
-    const int64_t j = tile * C + c;
-    const bool live = j < a.nsel;
-    const int64_t jj = live ? j : a.nsel - 1;  // columns past the end repeat the last one, unstored
+  const int64_t tile0 = (int64_t)blockIdx.x * a.tpc, tile1 = tile0 + a.tpc < ntiles ? tile0 + a.tpc : ntiles;
+  // frames t + T e of column tile * C + c, and what every frame is referred to
+  const auto load = [&](float2 (&u)[E], float2& x0, int64_t tile) {
+    const int64_t j = tile * C + c, jj = j < a.nsel ? j : a.nsel - 1;  // past the end: the last one, unstored
     const int64_t q = a.in_qsel ? a.in_qsel[jj] : jj;
-    float2 v[E];
     if constexpr (OUT == TIME_TILDE) {
       const float2* col = a.psi + (size_t)p * a.nf * a.in_nq + q;
-      const float2 x0 = a.ref[(size_t)p * a.in_nq + q];
+      x0 = a.ref[(size_t)p * a.in_nq + q];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int64_t n = t + T * e - a.f0;
-        v[e] = n >= 0 && n < a.nf ? col[(size_t)n * a.in_nq] - x0 : make_float2(0.f, 0.f);
+        u[e] = n >= 0 && n < a.nf ? col[(size_t)n * a.in_nq] : x0;
       }
     } else {
       const float2* col = a.psi + (size_t)p * F * a.in_nq + q;
-      const float2 x0 = col[0];
-      float2 sum = make_float2(0.f, 0.f);
+      x0 = col[0];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int n = t + T * e;
-        v[e] = !BLUE || n < F ? col[(size_t)n * a.in_nq] : x0;
+        u[e] = !BLUE || n < F ? col[(size_t)n * a.in_nq] : x0;
       }
+    }
+  };
+  float2 v[E], x0;
+  load(v, x0, tile0);
+  for (int64_t tile = tile0; tile < tile1; ++tile) {
+    const int64_t j = tile * C + c;
+    const bool live = j < a.nsel;
+    float2 next[E], next0;
+    if (TC::PREFETCH && tile + 1 < tile1) load(next, next0, tile + 1);
+    if constexpr (OUT == TIME_TILDE) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = v[e] - x0;
+    } else {
+      float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         v[e] = v[e] - x0;
@@ -147,7 +186,12 @@ __global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_
     if constexpr (OUT == TIME_DETECTOR) {
       if (live) {
 #pragma unroll
-        for (int e = 0; e < E; ++e) pair_add(hi[e], lo[e], v[e].x * v[e].x + v[e].y * v[e].y);
+        for (int e = 0; e < E; ++e) {
+          // FP32 pair: the exact errors of at most TIME_DET_TILES sums add up in lo
+          float err;
+          two_sum(hi[e], v[e].x * v[e].x + v[e].y * v[e].y, hi[e], err);
+          lo[e] += err;
+        }
       }
     } else if (live) {
       if constexpr (OUT == TIME_S) {
@@ -166,6 +210,13 @@ __global__ void __launch_bounds__(TimeCfg<N>::THREADS, TimeCfg<N>::MINB) k_time_
           else if (m < F) dst[(size_t)m * a.nsel] = cmul(v[e], __ldg(a.chirp + m));
         }
       }
+    }
+    if (TC::PREFETCH) {
+#pragma unroll
+      for (int e = 0; e < E; ++e) v[e] = next[e];
+      x0 = next0;
+    } else if (tile + 1 < tile1) {
+      load(v, x0, tile + 1);
     }
   }
   if constexpr (OUT == TIME_DETECTOR) {
@@ -201,16 +252,13 @@ int time_fft_length(int64_t F, bool* chirp) {
 
 namespace {
 
-template <int N>
-int64_t det_blocks(int64_t nsel) {
-  const int64_t tiles = (nsel + TimeCfg<N>::C - 1) / TimeCfg<N>::C;
-  return (tiles + TIME_DET_TILES - 1) / TIME_DET_TILES;
-}
-
 template <int N, int OUT, bool BLUE>
-cudaError_t launch_n(const TimeArgs& a, cudaStream_t st) {
-  using TC = TimeCfg<N>;
-  const int64_t gx = OUT == TIME_DETECTOR ? det_blocks<N>(a.nsel) : (a.nsel + TC::C - 1) / TC::C;
+cudaError_t launch_n(TimeArgs a, cudaStream_t st) {
+  using TC = TimeCfg<N, OUT, BLUE>;
+  const int64_t tiles = (a.nsel + TC::C - 1) / TC::C;
+  a.tpc = OUT == TIME_DETECTOR ? TIME_DET_TILES
+                               : (int)std::min<int64_t>(8, std::max<int64_t>(1, tiles * a.P / (8 * 152 * TC::MINB)));
+  const int64_t gx = (tiles + a.tpc - 1) / a.tpc;
   const int64_t gy = std::min<int64_t>(a.P, 65535), gz = (a.P + gy - 1) / gy;
   if (gx > 0x7fffffff || gz > 65535) return cudaErrorInvalidValue;
   auto* k = k_time_fft<N, OUT, BLUE>;
@@ -262,11 +310,9 @@ cudaError_t launch_time_fft(int n, const TimeArgs& a, int out, bool chirp, cudaS
   return cudaErrorInvalidValue;
 }
 
-int64_t time_det_blocks(int n, int64_t nsel) {
-#define TACAW_CALL(N) det_blocks<N>(nsel)
-  TACAW_TIME_DISPATCH(n, TACAW_CALL)
-#undef TACAW_CALL
-  return 0;
+int64_t time_det_blocks(int n, bool chirp, int64_t nsel) {
+  const int c = time_shape(n, TIME_DETECTOR, chirp).c * TIME_DET_TILES;
+  return (nsel + c - 1) / c;
 }
 
 }  // namespace
@@ -274,7 +320,7 @@ int64_t time_det_blocks(int n, int64_t nsel) {
 int64_t time_fft_parts(int64_t F, int64_t nsel) {
   bool chirp;
   const int n = time_fft_length(F, &chirp);
-  return n ? time_det_blocks(n, nsel) : 0;
+  return n ? time_det_blocks(n, chirp, nsel) : 0;
 }
 
 // S (full, or the spectrum image with REDUCE_DETECTOR) by FFT; the caller has checked
@@ -299,7 +345,7 @@ int spectrum_fft(tacaw_ctx* ctx, const float2* psi, int64_t P, int64_t F, const 
     if (rc != TACAW_OK) return rc;
   }
   const bool det = reduce == TACAW_REDUCE_DETECTOR;
-  const int64_t nparts = det ? time_det_blocks(n, io.nsel) : 0;
+  const int64_t nparts = det ? time_det_blocks(n, chirp, io.nsel) : 0;
   cudaError_t e;
   if (det && (e = sc.get(&a.part, (size_t)P * nparts * F)) != cudaSuccess) return cuda_err(ctx, e, "detector partial sums");
   const double pfq = (double)P * F * io.nsel;
