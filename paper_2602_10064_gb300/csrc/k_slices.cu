@@ -22,7 +22,7 @@ namespace tacaw {
 // Per-kernel variants of the FFT pass kernels, chosen per transform length by the autotuner
 // (paper_2602_10064_gb300/tune.py), which times every variant on GB300 and writes
 // tuning_table.h.  Variant bits: 1 = radix-8 plans (512 and 1024 points, 16 elements per
-// thread), 2 = 1.5 times as many resident threads per SM (fewer registers each), 4 = column
+// thread), 2 = 1.5 to 2 times as many resident threads per SM (fewer registers each), 4 = column
 // passes only: twice the columns per CTA, so that each load instruction covers whole 128-byte
 // lines, 8 = 32 elements per thread for the powers of two from 128 points (two-pass
 // transforms, about 170 registers).  TACAW_TUNE_FORCE=v builds every kernel as variant v (the
@@ -44,10 +44,12 @@ struct Tuned {
   static constexpr int EV = (V & 8) ? 1 : 0;
   static constexpr int PLAN = (V & 1) && !EV;
   static constexpr int WIDE = (COLUMN && (V & 4)) ? 1 : 0;
-  // resident CTAs per SM requested for a CTA of `threads`: `target` threads per SM (variant & 2:
-  // 1.5 times as many)
+  // resident CTAs per SM requested for a CTA of `threads`: `target` threads per SM; variant & 2: 1.5
+  // times as many, or twice where that makes no difference to the CTAs and in the spreading pass
   __host__ __device__ static constexpr int minb(int threads, int target) {
-    return ((V & 2) ? target * 3 / 2 : target) / threads > 1 ? ((V & 2) ? target * 3 / 2 : target) / threads : 1;
+    const int base = target / threads, more = target * 3 / 2 / threads, most = target * 2 / threads;
+    const int n = !(V & 2) ? base : K == K_SPLAT_ROW || more == base ? most : more;
+    return n > 1 ? n : 1;
   }
 };
 
@@ -116,12 +118,12 @@ __host__ __device__ constexpr int minb_of() {
   return Tuned<K, N>::minb(Cfg::THREADS, Cfg::TARGET);
 }
 
-// Barrier of one row transform: the group's own (warp, or named barrier over whole warps), or
-// the CTA barrier when a group of T threads is not made of whole warps (T = 48: 1152 points).
+// Barrier of one row transform: the group's own (warp, or named barrier over whole warps), or one of
+// the two groups that fill whole warps together (T = 48: 1152 points).
 template <int T>
 __device__ __forceinline__ auto group_sync(int g) {
   if constexpr (T <= 32 || T % 32 == 0) return GroupSync<T>{1 + g};
-  else return BlockSync{};
+  else return GroupSync<2 * T>{1 + g / 2};
 }
 
 // CTAs of a column pass: the in-band columns c < W only, C per CTA.  The padding columns up to Wp
