@@ -101,6 +101,21 @@ __global__ void k_intensity(const float2* __restrict__ pt, int64_t F, int64_t ns
   S[((size_t)p * F + m) * nq + q] = m == 0 ? 0.f : v.x * v.x + v.y * v.y;
 }
 
+// The same without a q list, four columns a thread in two 16-byte loads and one 16-byte store, for row
+// lengths that are multiples of four and 16-byte aligned buffers.  512 x 65536: 61 us, one column
+// a thread 103.
+__global__ void __launch_bounds__(256) k_intensity_x4(const float4* __restrict__ pt, int64_t F, int64_t n4,
+                                                      float4* __restrict__ S) {
+  const int64_t j = blockIdx.x * (int64_t)256 + threadIdx.x;
+  const int64_t m = blockIdx.y, p = blockIdx.z;
+  if (j >= n4) return;
+  const size_t row = (size_t)p * F + m;
+  const float4 a = pt[(row * n4 + j) * 2], b = pt[(row * n4 + j) * 2 + 1];
+  S[row * n4 + j] = m == 0 ? make_float4(0.f, 0.f, 0.f, 0.f)
+                           : make_float4(a.x * a.x + a.y * a.y, a.z * a.z + a.w * a.w, b.x * b.x + b.y * b.y,
+                                         b.z * b.z + b.w * b.w);
+}
+
 // SI[p][m] = sum_j |psi~[p][m][j]|^2 (FP64, fixed reduction tree), 0 at m = 0.
 __global__ void __launch_bounds__(256) k_intensity_detector(const float2* __restrict__ pt, int64_t F, int64_t nsel,
                                                             float* __restrict__ SI) {
@@ -206,8 +221,12 @@ int tacaw_intensity(tacaw_ctx* ctx, const float* psi_tilde, int64_t P, int64_t F
       if (e != cudaSuccess) return cuda_err(ctx, e, "cudaMemsetAsync");
     }
     ProfScope ps(ctx, "intensity", st, (double)P * F * n_sel * 12, (double)P * F * n_sel * 3);
-    k_intensity<<<dim3((unsigned)((n_sel + 255) / 256), (unsigned)F, (unsigned)P), 256, 0, st>>>(pt, F, n_sel, q_sel,
-                                                                                                nq, S_out);
+    if (!q_sel && n_sel % 4 == 0 && ((uintptr_t)psi_tilde | (uintptr_t)S_out) % 16 == 0)
+      k_intensity_x4<<<dim3((unsigned)((n_sel / 4 + 255) / 256), (unsigned)F, (unsigned)P), 256, 0, st>>>(
+          reinterpret_cast<const float4*>(psi_tilde), F, n_sel / 4, reinterpret_cast<float4*>(S_out));
+    else
+      k_intensity<<<dim3((unsigned)((n_sel + 255) / 256), (unsigned)F, (unsigned)P), 256, 0, st>>>(pt, F, n_sel, q_sel,
+                                                                                                  nq, S_out);
   } else {
     ProfScope ps(ctx, "intensity_detector", st, (double)P * F * n_sel * 8, (double)P * F * n_sel * 4);
     k_intensity_detector<<<dim3((unsigned)F, (unsigned)P), 256, 0, st>>>(pt, F, n_sel, S_out);
