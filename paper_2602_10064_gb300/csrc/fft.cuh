@@ -292,6 +292,13 @@ struct FftPlan {
   static constexpr int T = N / E;
 };
 
+// Asynchronous 8-byte copy global -> shared (completes at cp_async_wait_all of the same thread).
+__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem_src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // Barrier of the whole CTA, for transforms whose threads interleave with other transforms'.
 struct BlockSync {
   __device__ __forceinline__ void operator()() const { __syncthreads(); }

@@ -937,13 +937,6 @@ struct SliceRowSmem {
   static constexpr int BYTES = SliceRowCfg<NX, TF>::SMEM + SliceRowCfg<NX, TF>::G * NX * (int)sizeof(float2);
 };
 
-// Asynchronous 8-byte copy global -> shared (completes at cp_async_wait_all of the same thread).
-__device__ __forceinline__ void cp_async8(void* smem_dst, const void* gmem_src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(smem_dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d), "l"(gmem_src) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
 // Most waves that one CTA of the slice column pass takes through its columns.  256 points, 2304 waves,
 // 16 elements a thread: 2.97 ms for 8 slices with the loop; 4.16 with 32 elements, which spill in it.
 constexpr int SLICE_COL_WAVES = 8;

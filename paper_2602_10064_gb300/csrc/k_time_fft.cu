@@ -67,9 +67,16 @@ struct TimeCfg {
   static constexpr TimeShape SHAPE = time_shape(N, OUT, BLUE);
   static constexpr int E = SHAPE.e, T = N / E, C = SHAPE.c, THREADS = T * C, MINB = SHAPE.minb;
   static constexpr int SH = E == 32 ? 5 : 0;
-  static constexpr int SMEM = (N + (SH ? N >> SH : 0)) * C * (int)sizeof(float2);
-  // the spectrum image keeps its running sums in those registers
-  static constexpr bool PREFETCH = SHAPE.prefetch && OUT != TIME_DETECTOR;
+  static constexpr int SCRATCH = (N + (SH ? N >> SH : 0)) * C * (int)sizeof(float2), TILE = N * C * (int)sizeof(float2);
+  // The next tile comes into registers where they are free.  The spectrum image keeps its running sums
+  // in them and the chirp-z forms need them; there it comes by cp.async into shared memory (each thread
+  // copies and reads its own elements) for the short transforms and for S through 1024 points: ps an
+  // element without -> with it, image and chirp-z S at 32 points 3.53 -> 3.25 and 9.49 -> 7.33, 128
+  // points 3.06 -> 2.73 and 7.57 -> 6.95, chirp-z S at 1024 11.2 -> 10.1.  At 256 and 512 points the
+  // second buffer costs more than it gives (image 2.72 -> 2.89 and 3.29 -> 5.26).
+  static constexpr bool ASYNC = (OUT == TIME_DETECTOR || BLUE) && (N <= 128 || (N == 1024 && OUT != TIME_DETECTOR));
+  static constexpr bool PREFETCH = SHAPE.prefetch && OUT != TIME_DETECTOR && !BLUE;
+  static constexpr int SMEM = SCRATCH + (ASYNC ? TILE : 0);
 };
 
 struct TimeArgs {
@@ -136,16 +143,44 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
       }
     }
   };
+  // the same into this thread's slots of the tile buffer; x0 into a register
+  float2* slots = reinterpret_cast<float2*>(smraw + TC::SCRATCH) + threadIdx.x;  // [E][THREADS]
+  const auto fetch = [&](float2& x0, int64_t tile) {
+    const int64_t j = tile * C + c, jj = j < a.nsel ? j : a.nsel - 1;
+    const int64_t q = a.in_qsel ? a.in_qsel[jj] : jj;
+    const bool part = OUT == TIME_TILDE;
+    const float2* col = a.psi + (size_t)p * (part ? a.nf : (int64_t)F) * a.in_nq + q;
+    x0 = part ? a.ref[(size_t)p * a.in_nq + q] : col[0];
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int64_t n = t + T * e - (part ? a.f0 : 0);
+      if (part ? n >= 0 && n < a.nf : !BLUE || n < F)
+        cp_async8(slots + TC::THREADS * e, col + (size_t)n * a.in_nq);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  const auto collect = [&](float2 (&u)[E], float2 x0) {
+    cp_async_wait_all();
+#pragma unroll
+    for (int e = 0; e < E; ++e) {
+      const int64_t n = t + T * e - (OUT == TIME_TILDE ? a.f0 : 0);
+      const bool in = OUT == TIME_TILDE ? n >= 0 && n < a.nf : !BLUE || n < F;
+      u[e] = in ? slots[TC::THREADS * e] : x0;
+    }
+  };
   float2 v[E], x0;
-  load(v, x0, tile0);
+  if (TC::ASYNC) fetch(x0, tile0);
+  else load(v, x0, tile0);
   for (int64_t tile = tile0; tile < tile1; ++tile) {
     const int64_t j = tile * C + c;
     const bool live = j < a.nsel;
     float2 next[E], next0;
+    if (TC::ASYNC) collect(v, x0);
     if (TC::PREFETCH && tile + 1 < tile1) load(next, next0, tile + 1);
     if constexpr (OUT == TIME_TILDE) {
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = v[e] - x0;
+      if (TC::ASYNC) __syncthreads();  // every slot has been read
     } else {
       float2 sum = make_float2(0.f, 0.f);
 #pragma unroll
@@ -170,6 +205,8 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = !BLUE || t + T * e < F ? v[e] - mean : make_float2(0.f, 0.f);
     }
+    // (both branches have passed a barrier after the slots were read)
+    if (TC::ASYNC && tile + 1 < tile1) fetch(x0, tile + 1);
     if constexpr (BLUE) {
 #pragma unroll
       for (int e = 0; e < E; ++e) {
@@ -215,7 +252,7 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = next[e];
       x0 = next0;
-    } else if (tile + 1 < tile1) {
+    } else if (!TC::ASYNC && tile + 1 < tile1) {
       load(v, x0, tile + 1);
     }
   }
