@@ -40,8 +40,10 @@ template <int SIGN>
 __device__ __forceinline__ float2 add_si(float2 a, float2 b) {
   return SIGN < 0 ? make_float2(a.x + b.y, a.y - b.x) : make_float2(a.x - b.y, a.y + b.x);
 }
+// Which of the two products of a sum is rounded is left to the compiler otherwise, and differed between
+// the forms of one kernel (looped or not).
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
-  return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+  return make_float2(fmaf(-a.y, b.y, a.x * b.x), fmaf(a.y, b.x, a.x * b.y));
 }
 __device__ __forceinline__ float2 conjf2(float2 a) { return make_float2(a.x, -a.y); }
 
