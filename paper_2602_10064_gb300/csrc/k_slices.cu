@@ -72,24 +72,33 @@ __host__ __device__ constexpr int floor_pow2(int x) {
 // elements per thread need about 170 registers, so those CTAs are smaller and the SM holds
 // 384 instead of 512 threads (TARGET).
 // EV = 1: 32 elements per thread (two-pass transforms) for the powers of two from 128 points.
-template <int N, int EV = 0>
+// SMALL and LARGE, threads per CTA with up to 16 elements each and with more: the spreading pass takes 256
+// and 192, to share its candidate tables over more rows, the others 64 and 192: small CTAs keep the phases
+// of an SM's warps apart.  256-point slice row pass of a probe scan, 160 launches: 48.3 ms with 256
+// threads, 45.7 with 128, 44.3 with 64.  The slice row pass takes 96 where a row lies in half a warp (512
+// points 4.01 ps a point with 192, 3.76 with 96; 384 points 4.53, 4.40); not above that, where it has to
+// synchronise several warps (768 points 4.33, 4.43; 1152 points 4.81, 4.90).
+template <int N, int EV = 0, int SMALL = 64, int LARGE = 192>
 struct RowCfg {
   static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N, TACAW_ROW_E>::E;
   static constexpr int T = N / E;
   static constexpr int TARGET = E >= 24 ? 384 : 512;
-  static constexpr int G0 = (TARGET / 2) / T;
+  static constexpr int G0 = (E < 24 ? SMALL : T < 32 ? LARGE : 192) / T;
   static constexpr int G = G0 > 32 ? 32 : (G0 < 1 ? 1 : floor_pow2(G0));  // rows per CTA
   static constexpr int THREADS = G * T;
   static constexpr int SMEM = G * row_smem_stride<N, E>() * (int)sizeof(float2);
 };
 
-// Column passes: C columns per CTA (about 256 threads; WIDE doubles C, about 512 threads).
+// Column passes: C columns per CTA (WIDE doubles C).  With 8 or 16 elements a thread, 128 threads but
+// at least 16 columns (whole 128-byte lines) where 256 threads hold them: 64 points 5.85 -> 4.94 and
+// 128 points 3.23 -> 2.97 ps a point in the slice pass; 256 points lose 5% with 8 columns.
 template <int N, int WIDE = 0, int EV = 0>
 struct ColCfg {
   static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N, TACAW_COL_E>::E;
   static constexpr int T = N / E;
   static constexpr int TARGET = E >= 24 ? 384 : 512;
-  static constexpr int C0 = ((TARGET / 2) << WIDE) / T;
+  static constexpr int FULL = TARGET / 2 / T, HALF = TARGET / 4 / T;
+  static constexpr int C0 = (E >= 24 || FULL <= 16 ? FULL : HALF < 16 ? 16 : HALF) << WIDE;
   static constexpr int C = C0 > 32 ? 32 : (C0 < 4 ? 4 : floor_pow2(C0));  // columns per CTA (divides Wp)
   static constexpr int THREADS = C * T;
   // padding of the interleaved columns: pays only with 32 elements per thread (with 8 columns of 1152
@@ -99,14 +108,14 @@ struct ColCfg {
 };
 
 // The configuration of each pass kernel; a kernel and its launcher name the same alias.
-template <int N> using SplatCfg = RowCfg<N, Tuned<K_SPLAT_ROW, N>::EV>;
+template <int N> using SplatCfg = RowCfg<N, Tuned<K_SPLAT_ROW, N>::EV, 256>;
 template <int N> using PotOutCfg = RowCfg<N, Tuned<K_ROW_POT_OUT, N>::EV>;
 template <int N> using RowVtCfg = RowCfg<N, Tuned<K_ROW_VT, N>::EV>;
 template <int N> using RowToutCfg = RowCfg<N, Tuned<K_ROW_TOUT, N>::EV>;
 template <int N> using ProbeRowCfg = RowCfg<N, Tuned<K_PROBE_ROW, N>::EV>;
 // one probe (the compact t, TF) and several (the full t) have different loops: tuned apart
 template <bool TF> __host__ __device__ constexpr int slice_row_id() { return TF ? K_SLICE_ROW : K_SLICE_ROW_SCAN; }
-template <int N, bool TF> using SliceRowCfg = RowCfg<N, Tuned<slice_row_id<TF>(), N>::EV>;
+template <int N, bool TF> using SliceRowCfg = RowCfg<N, Tuned<slice_row_id<TF>(), N>::EV, 64, 96>;
 template <int N> using ColPotCfg = ColCfg<N, Tuned<K_COL_POT, N>::WIDE, Tuned<K_COL_POT, N>::EV>;
 template <int N> using ColTCfg = ColCfg<N, Tuned<K_COL_T, N>::WIDE, Tuned<K_COL_T, N>::EV>;
 template <int N> using ProbeColCfg = ColCfg<N, Tuned<K_PROBE_COL, N>::WIDE, Tuned<K_PROBE_COL, N>::EV>;
@@ -934,7 +943,10 @@ __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW,
 // Shared memory of the slice row pass: the FFT scratch, plus (TF) one stashed t row per group.
 template <int NX, bool TF>
 struct SliceRowSmem {
-  static constexpr int BYTES = SliceRowCfg<NX, TF>::SMEM + SliceRowCfg<NX, TF>::G * NX * (int)sizeof(float2);
+  // up to 16 elements a thread, the transmission row of several probes stays in registers
+  static constexpr bool TREG = !TF && SliceRowCfg<NX, TF>::E <= 16;
+  static constexpr int BYTES =
+      SliceRowCfg<NX, TF>::SMEM + (TREG ? 0 : SliceRowCfg<NX, TF>::G * NX * (int)sizeof(float2));
 };
 
 // Most waves that one CTA of the slice column pass takes through its columns.  256 points, 2304 waves,
@@ -942,7 +954,7 @@ struct SliceRowSmem {
 constexpr int SLICE_COL_WAVES = 8;
 // Most probes of a frame that one CTA of the slice row pass takes through its rows.  One probe a CTA
 // copied the transmission row (60% of the pass's reads) once for every probe and waited for every
-// wave's row; with eight, 256 points x 2048 waves take 300 us instead of 360.
+// wave's row; with eight, 256 points x 2048 waves take 280 us instead of 360.
 constexpr int SLICE_ROW_PROBES = 8;
 
 // MB >= 0: the band's half-width, fixed at compile time (the standard 2/3 band of a square
@@ -973,13 +985,14 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
     store_row_compact<NX>(v, Bpsi + ((size_t)bi * ny + y) * b.Wp, b, t);
     return;
   }
-  // The transmission row goes to a shared-memory stash before it is used; each thread writes
-  // and rereads only its own positions, so no barrier is needed.  TF: t is inverse-transformed
-  // first (only one row of the wave is then live in registers).  Otherwise the full t row is
-  // copied asynchronously at once, so its load overlaps the wave's load and inverse transform.
+  // The probes p0 .. p1 - 1 of this frame share the transmission row.  TF: it is inverse-transformed
+  // first and stashed in shared memory (only one row of the wave is then live in registers; each thread
+  // rereads only its own positions, so no barrier is needed), the wave's row loading meanwhile.  TREG: it
+  // stays in registers; the shared-memory pipe, three quarters busy with the exchanges, is the pass's
+  // bound, and this drops a read per element (256 points: 45.7 -> 44.9 ms).  Otherwise it is copied
+  // asynchronously into the stash, and the next probe's row loads while this one's is transformed.
+  constexpr bool TREG = SliceRowSmem<NX, TF>::TREG;
   float2* tst = reinterpret_cast<float2*>(smraw + RC::SMEM) + g * NX;
-  // The probes p0 .. p1 - 1 of this frame share the stashed row: the row of the next probe's wave is
-  // loaded while this one's is transformed.
   const auto load = [&](float2 (&u)[E], int p) {
     if (!FIRST) {
       load_row<NX, MB>(u, Apsi + ((size_t)(p * nfc + fl) * ny + y) * b.Wp, b, t);
@@ -992,8 +1005,10 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
       for (int e = 0; e < E; ++e) u[e] = src[t + T * e];
     }
   };
+  const float2* trow = ttab + ((size_t)(fl * S + s) * ny + y) * NX;
   float2 next[E];
-  if (TF) {
+  float2 tr[TREG ? E : 1];
+  if constexpr (TF) {
     load_row<NX, MB>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
     load(next, p0);
     fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
@@ -1001,27 +1016,35 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
     for (int e = 0; e < E; ++e) tst[t + T * e] = v[e];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = next[e];
+  } else if constexpr (TREG) {
+    load(v, p0);
+#pragma unroll
+    for (int e = 0; e < E; ++e) tr[e] = trow[t + T * e];
   } else {
-    const float2* trow = ttab + ((size_t)(fl * S + s) * ny + y) * NX;
 #pragma unroll
     for (int e = 0; e < E; ++e) cp_async8(tst + t + T * e, trow + t + T * e);
     asm volatile("cp.async.commit_group;" ::: "memory");
     load(v, p0);
   }
   for (int p = p0; p < p1; ++p) {
-    if (!TF && p + 1 < p1) load(next, p + 1);
+    if (!TF && !TREG && p + 1 < p1) load(next, p + 1);
     if (!FIRST) fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
-    if (!TF) cp_async_wait_all();
+    if (!TF && !TREG) cp_async_wait_all();
 #pragma unroll
     for (int e = 0; e < E; ++e) {
-      if (FIRST && PLANE) v[e] = plane_amp * tst[t + T * e];
-      else v[e] = cmul(v[e], tst[t + T * e]);
+      const float2 tv = TREG ? tr[TREG ? e : 0] : tst[t + T * e];
+      if (FIRST && PLANE) v[e] = plane_amp * tv;
+      else v[e] = cmul(v[e], tv);
     }
     fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
     store_row<NX, MB>(v, Bpsi + ((size_t)(p * nfc + fl) * ny + y) * b.Wp, b, t);
     if (TF) return;  // one probe
+    if (!TREG) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) v[e] = next[e];
+      for (int e = 0; e < E; ++e) v[e] = next[e];
+    } else if (p + 1 < p1) {
+      load(v, p + 1);
+    }
   }
 }
 
