@@ -7,8 +7,9 @@
 // psi~ itself (one process's share of a frame-sharded transform).  The stack is read once and the
 // result written once; the dense forms of the transform read it two or three times, write a
 // residual or split operands and do O(F) work per element where this does O(log F).  1024 frames x
-// 65536 q: 14.6 ms dense FP32, 0.31 ms here (2.5 TB/s; the loads of a CTA do not overlap its own
-// transform); a partial transform of 256 of 512 frames: 2.04 ms, 0.16 ms.
+// 65536 q: 14.6 ms dense FP32, 0.23 ms here (3.5 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
+// 0.17 ms.  Bound by latency: no pipe is above half of its rate (shared memory 48%, FP32 47%, DRAM 42% in
+// the image at 256 frames; 51% of the issue slots by the 8 warps that fit in the chirp-z form at 1024).
 //
 // Mean: every frame is first referred to the column's first frame, r1_n = psi_n - psi_0, which
 // rounds at the scale of the fluctuation (the difference of two nearly equal floats is exact), then
@@ -100,6 +101,33 @@ struct TimeArgs {
 // Column tiles one CTA of the spectrum image adds up before it stores its partial sums.  Fixed, so
 // that the order of the sums does not depend on how many probes a call holds.
 constexpr int TIME_DET_TILES = 8;
+
+// The sums over the C columns of a CTA, C neighbouring lanes of a warp: n bins a lane as FP32 pairs.  In
+// each step two lanes O apart add theirs; while n is even each of the two keeps one half of the bins
+// (from e0 on), then both keep all and one of them writes.  In FP64 (three operations an element on a
+// pipe of two results a clock) these sums took a third of the pass at 256 frames; image of 32 probes, 256
+// frames 465 -> 435 us, ps an element at 32, 192, 512, 2048 frames 3.23 -> 2.56, 3.52 -> 2.67, 3.17 -> 2.73,
+// 5.88 -> 5.15.
+__host__ __device__ constexpr int kept_bins(int n, int c) { return c == 1 ? n : kept_bins(n % 2 ? n : n / 2, c / 2); }
+template <int n, int O>
+__device__ __forceinline__ void column_pairs(float* hi, float* lo, int c, int& e0, bool& writer) {
+  if constexpr (O > 0) {
+    constexpr int KEEP = n % 2 ? n : n / 2;
+    const bool up = c & O;
+#pragma unroll
+    for (int e = 0; e < KEEP; ++e) {
+      const int other = n % 2 ? e : e + KEEP;
+      const float h = up ? hi[other] : hi[e], l = up ? lo[other] : lo[e];
+      const float gh = up ? hi[e] : hi[other], gl = up ? lo[e] : lo[other];
+      float err;
+      two_sum(h, __shfl_xor_sync(0xffffffffu, gh, O), hi[e], err);
+      lo[e] = __fadd_rn(__fadd_rn(l, __shfl_xor_sync(0xffffffffu, gl, O)), err);
+    }
+    if (n % 2) writer = writer && !up;
+    else if (up) e0 += KEEP;
+    column_pairs<KEEP, O / 2>(hi, lo, c, e0, writer);
+  }
+}
 
 template <int N, int OUT, bool BLUE>
 __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT, BLUE>::MINB) k_time_fft(const TimeArgs a) {
@@ -257,17 +285,17 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
     }
   }
   if constexpr (OUT == TIME_DETECTOR) {
-    // over the columns, in FP64 and in an order fixed per bin
-    double* red = reinterpret_cast<double*>(smraw);  // [N][C]
-    __syncthreads();
+    // over the columns, still as pairs and in an order fixed per bin
+    int e0 = 0;
+    bool writer = true;
+    column_pairs<E, C / 2>(hi, lo, c, e0, writer);
+    if (writer) {
 #pragma unroll
-    for (int e = 0; e < E; ++e) red[(t + T * e) * C + c] = (double)hi[e] + (double)lo[e];
-    __syncthreads();
-    for (int m = threadIdx.x; m < F; m += TC::THREADS) {
-      double s = 0.0;
-#pragma unroll
-      for (int k = 0; k < C; ++k) s += red[m * C + (k + m) % C];
-      a.part[((size_t)p * gridDim.x + blockIdx.x) * F + m] = s;
+      for (int e = 0; e < kept_bins(E, C); ++e) {
+        const int m = t + T * (e0 + e);
+        if (m < F)  // a sum past the largest float stays infinite
+          a.part[((size_t)p * gridDim.x + blockIdx.x) * F + m] = (double)hi[e] + (isinf(hi[e]) ? 0.0 : (double)lo[e]);
+      }
     }
   }
 }
