@@ -10,8 +10,8 @@ import workloads
 pytestmark = pytest.mark.gpu
 
 
-# rows of 64 and 96 points hold 8 and 12 elements a thread, those of 384, 512 and 768 points 24 or 32;
-# 5 x 5 probes split unevenly; one probe: the compact transmission row and the column pass alone
+# rows of 64, 128 and 256 points hold 8 or 16 elements a thread, those of 96, 384, 512 and 768 points 24 or
+# 32; 5 x 5 probes split unevenly; one probe: the compact transmission row and the column pass alone
 @pytest.mark.parametrize("grid,side,frames,chunk", [(64, 5, 36, 1), (96, 5, 24, 1), (128, 3, 48, 2), (256, 5, 10, 1),
                                                     (384, 5, 6, 1), (512, 3, 8, 1), (768, 3, 6, 1), (128, 1, 400, 40)])
 def test_looped_launches_give_the_same_bits(grid, side, frames, chunk):
