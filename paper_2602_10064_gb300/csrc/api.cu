@@ -913,8 +913,10 @@ int slices(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const float2* t, 
   for (int s = s0; s < s0 + sb; ++s) {
     const bool last = s == S - 1;
     {
-      const double in = s > 0 ? W8 : (psi0 ? 8.0 * p.nx : 0.0), tin = tfused ? W8 : 8.0 * p.nx;
-      ProfScope ps(ctx, "slice_row", sc.st, rows * (in + tin + W8), rows * ((s > 0 ? 2 : 1) + (tfused ? 1 : 0)) * fx);
+      // a frame's transmission rows are one read for all its probes, a probe's psi0 one for all frames
+      const double bytes = rows * W8 + (s > 0 ? rows * W8 : psi0 ? rows / nfc * 8.0 * p.nx : 0.0) +
+                           rows / P * (tfused ? W8 : 8.0 * p.nx);
+      ProfScope ps(ctx, "slice_row", sc.st, bytes, rows * ((s > 0 ? 2 : 1) + (tfused ? 1 : 0)) * fx);
       CK(launch_slice_row(geo, g->band, s == 0, psi0 == nullptr, tfused, Apsi, psi0, t, t_slices, s - t_first, P,
                           nfc, plane_amp, Bpsi, (int)ctx->static_band, sc.st));
     }
@@ -962,7 +964,9 @@ struct RunTiling {
 RunTiling run_tiling(const tacaw_ctx* ctx, const tacaw_params& p, const GeoCache* g, int P, int64_t F) {
   const size_t nq = (size_t)p.nx * p.ny, plane = (size_t)p.ny * g->band.Wp, cap = kChunkCap;
   const int S = p.n_slices;
-  const size_t per_slice = nq * 8 + plane * 8 * (g->npair + 3), wave = (size_t)P * plane * 16;
+  // t (full, and At, or compact), Bp, Ap and Bt
+  const size_t per_slice = (use_compact_t(p, P) ? 0 : nq * 8) + plane * 8 * (g->npair + 3);
+  const size_t wave = (size_t)P * plane * 16;
   const int64_t rows = ctx->min_wave_rows > 0 ? ctx->min_wave_rows : kMinWaveRows;
   int64_t want = std::min<int64_t>(F, (rows + (int64_t)P * p.ny - 1) / ((int64_t)P * p.ny));
   if (ctx->max_chunk_frames > 0) want = std::min<int64_t>(want, ctx->max_chunk_frames);
@@ -970,11 +974,16 @@ RunTiling run_tiling(const tacaw_ctx* ctx, const tacaw_params& p, const GeoCache
   if ((size_t)want * (S * per_slice + wave) > cap) {
     const size_t room = cap / (size_t)want;
     sb = room > wave ? (int)std::min<size_t>(S, std::max<size_t>(1, (room - wave) / per_slice)) : 1;
+    // one species: a pair of slices is one potential transform, which a block that cuts the pair
+    // repeats.  Whole pairs, though a launch then holds fewer waves: 1152 points, 54 slices, 200
+    // frames 370 -> 301 ms (39 frames x 1 slice -> 29 x 2), 1024 points, 256 frames 100.5 -> 82.8
+    if (g->nslot == 1) sb = std::min(S, std::max(2, sb & ~1));
   }
   if (ctx->max_slice_block > 0) sb = (int)std::min<int64_t>(sb, ctx->max_slice_block);
   int64_t c = chunk_frames(F, sb * per_slice + wave, cap);
   if (ctx->max_chunk_frames > 0) c = std::min<int64_t>(c, ctx->max_chunk_frames);
-  return RunTiling{c, sb};
+  const int64_t chunks = (F + c - 1) / c;
+  return RunTiling{(F + chunks - 1) / chunks, sb};  // even chunks
 }
 
 // Probe blocks of a run.  Every probe needs its exit-wave stack (F in-band points, compact)

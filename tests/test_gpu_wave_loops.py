@@ -33,3 +33,25 @@ def test_looped_launches_give_the_same_bits(grid, side, frames, chunk):
         ctx.check()
         assert float(whole.abs().max()) > 0
         assert torch.equal(whole, parts)
+
+
+@pytest.mark.parametrize("block", [1, 3])
+def test_blocks_of_whole_slice_pairs_give_the_same_bits(block):
+    # one species and more frames than a block of all 5 slices has room for: blocks of slices 2, 2, 1, against
+    # blocks that cut the pairs
+    import __graft_entry__
+    __graft_entry__.build()
+    import torch
+
+    import paper_2602_10064_gb300 as T
+    w = workloads.diamond_si(n_frames=130, grid=512, n_slices=5, seed=5)
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).cuda()
+    with T.Context(0) as ctx:
+        ctx.load_form_factors(w.form_Z, w.form_coef)
+        p, pr, pos, Z = T.params_of(w), T.probe_of(w), dev(w.pos), dev(w.Z)
+        pairs = ctx.run(p, pos, Z, pr, precision=T.DFT_FP32)
+        ctx.set_option("max_slice_block", block)
+        cut = ctx.run(p, pos, Z, pr, precision=T.DFT_FP32)
+        ctx.check()
+        assert float(pairs.abs().max()) > 0
+        assert torch.equal(pairs, cut)
