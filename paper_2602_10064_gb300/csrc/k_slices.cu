@@ -254,6 +254,8 @@ __device__ __forceinline__ int slice_of(double z, const BinGeom& g) {
   return s;
 }
 
+// The index stays in [0, n) for every x: 0 where x is not finite (its fraction is NaN, which the spreading
+// kernel takes as out of reach: the atom adds nothing) or too far out for FP64 to wrap.
 __device__ __forceinline__ void grid_coord(double x, double L, double per_len, int n, int& i0, float& fr) {
   const double u = __dmul_rn(wrap_cell(x, L), per_len);
   double fl = floor(u);
@@ -261,7 +263,7 @@ __device__ __forceinline__ void grid_coord(double x, double L, double per_len, i
   double f = __dsub_rn(u, fl);
   if (i >= n) { i -= n; }
   if (i < 0) { i += n; }
-  i0 = i;
+  i0 = i >= 0 && i < n ? i : 0;
   fr = (float)f;
 }
 
