@@ -635,9 +635,7 @@ namespace tacaw {
 
 // Form-factor slot of every atom.  Z on the device is mapped there; what becomes of an unknown
 // species depends on the caller: device_check reports it through the context's status word
-// (tacaw_check), else through a flag of this call that species_verdict reads once the call's work is
-// enqueued, so the device does not wait for the host either way.  Z on the host is checked here
-// (EINVAL).
+// (tacaw_check), else a SpeciesVerdict reads it.  Z on the host is checked here (EINVAL).
 int make_slots(tacaw_ctx* ctx, const int32_t* Z, int64_t A, bool z_on_device, bool device_check, Scratch& sc,
                int8_t** d_slot) {
   if (z_on_device) {
@@ -677,18 +675,36 @@ int make_slots(tacaw_ctx* ctx, const int32_t* Z, int64_t A, bool z_on_device, bo
   return TACAW_OK;
 }
 
-// Result of the species check of make_slots without device_check: waits for the mapping only.
-int species_verdict(tacaw_ctx* ctx, const int32_t* Z, int64_t A, cudaStream_t st) {
-  CK(cudaEventSynchronize(ctx->species_event));
-  if (!*ctx->species_flag) return TACAW_OK;
-  std::vector<int32_t> hz(A);
-  CK(cudaMemcpyAsync(hz.data(), Z, sizeof(int32_t) * A, cudaMemcpyDeviceToHost, st));
-  CK(cudaStreamSynchronize(st));
-  for (int64_t j = 0; j < A; ++j)
-    if (std::find(ctx->ffZ.begin(), ctx->ffZ.end(), hz[j]) == ctx->ffZ.end())
-      return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, hz[j]);
-  return set_err(ctx, TACAW_EINVAL, "an atom's Z is not in the form-factor table");
-}
+// The species check of make_slots without device_check: get() waits for the mapping alone (once), EINVAL
+// if an atom's Z is not in the table.  A call asks before it enqueues the first kernel that writes its
+// output, with the kernels of its scratch already running, and again before it returns, whatever
+// ended it, so that no copy into the context's flag outlives it.
+struct SpeciesVerdict {
+  tacaw_ctx* ctx;
+  const int32_t* Z;
+  int64_t A;
+  cudaStream_t st;
+  bool known = false;
+  int rc = TACAW_OK;
+  int get() {
+    if (!known) rc = wait();
+    known = true;
+    return rc;
+  }
+
+ private:
+  int wait() {
+    CK(cudaEventSynchronize(ctx->species_event));
+    if (!*ctx->species_flag) return TACAW_OK;
+    std::vector<int32_t> hz(A);
+    CK(cudaMemcpyAsync(hz.data(), Z, sizeof(int32_t) * A, cudaMemcpyDeviceToHost, st));
+    CK(cudaStreamSynchronize(st));
+    for (int64_t j = 0; j < A; ++j)
+      if (std::find(ctx->ffZ.begin(), ctx->ffZ.end(), hz[j]) == ctx->ffZ.end())
+        return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, hz[j]);
+    return set_err(ctx, TACAW_EINVAL, "an atom's Z is not in the form-factor table");
+  }
+};
 
 // Binned atoms of frames [0, nf): per-(frame, slice) lists, then the row-sorted copy with the
 // offsets of every block of SPREAD_YB grid rows that the spreading pass reads.
@@ -1200,16 +1216,19 @@ int tacaw_build_potential(tacaw_ctx* ctx, const tacaw_params* params, const floa
   const Geo geo{p.nx, p.ny, ctx->tw};
   const size_t plane = (size_t)p.ny * g->band.Wp;
   const int64_t chunk = chunk_frames(nf, p.n_slices * plane * 8 * (g->npair + 1), (size_t)1 << 30);
-  TRY_RC(potential_chunks(ctx, p, g, pos, slots, n_atoms, nf, chunk, p.n_slices, sc,
-                          [&](int64_t f0, int nfc, const PotPlanes& pp) {
+  SpeciesVerdict species{ctx, Z, n_atoms, st};
+  const int rc = potential_chunks(ctx, p, g, pos, slots, n_atoms, nf, chunk, p.n_slices, sc,
+                                  [&](int64_t f0, int nfc, const PotPlanes& pp) {
+    TRY_RC(species.get());
     ProfScope ps(ctx, "row_pot_out", st,
                  (double)pp.planes * p.ny * 8.0 * g->band.W + (double)nfc * p.n_slices * p.ny * 4.0 * p.nx,
                  (double)pp.planes * p.ny * 5.0 * p.nx * std::log2((double)p.nx));
     CK(launch_row_pot_out(geo, g->band, pp.Ap, pp.planes, pp.sp, 0, 0.f,
                           V_out + (size_t)f0 * p.n_slices * p.ny * p.nx, nullptr, (int)ctx->static_band, st));
     return TACAW_OK;
-  }));
-  return species_verdict(ctx, Z, n_atoms, st);
+  });
+  TRY_RC(species.get());
+  return rc;
 }
 
 int tacaw_transmission(tacaw_ctx* ctx, const tacaw_params* params, const float* V, int64_t nf, float* t_out,
