@@ -686,7 +686,7 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
 // the second in the imaginary part, so both take one inverse transform (and one spreading and one
 // column pass before it): three transforms per two rows instead of four here.  1152 points x 54 slices
 // x 20 frames: splat_row 4.10 -> 2.61 ms, col_pot 5.90 -> 3.05, this 7.08 -> 5.95.  A slice
-// without atoms is zero exactly, whatever its partner rounds to.
+// without atoms is zero exactly, whatever its partner rounds to.  Modes 1 and 2 only (potential_block).
 template <int NX, bool PAIR, int MB = -1>
 __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT, NX, PotOutCfg<NX>>())
     k_row_pot_out(Geo geo, Band b, const float2* __restrict__ Ap, int nbatch, SlicePairs sp, int mode, float sigma,
@@ -717,10 +717,10 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
   for (int e = 0; e < E; ++e) im[e] = v[e].y;
 #pragma unroll 1
   for (; s < s_end; ++s) {
-    float scale = 1.f;
+    bool atoms = true;
     if (PAIR) {
       const int* bo = sp.boffs + ((size_t)f * sp.S + s) * (ny / SPREAD_YB + 1);
-      scale = bo[ny / SPREAD_YB] > bo[0] ? 1.f : 0.f;
+      atoms = bo[ny / SPREAD_YB] > bo[0];
       if (s > s_first) {
 #pragma unroll
         for (int e = 0; e < E; ++e) v[e].x = im[e];
@@ -728,16 +728,15 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
     }
     const size_t plane = PAIR ? (size_t)f * sp.sb + (s - sp.s0) : (size_t)bi;
     const size_t row = (plane * ny + y) * NX;
-    if (mode == 0) {
+    if (!PAIR && mode == 0) {
 #pragma unroll
-      for (int e = 0; e < E; ++e) V[row + t + T * e] = PAIR ? scale * v[e].x : v[e].x;
+      for (int e = 0; e < E; ++e) V[row + t + T * e] = v[e].x;
       continue;
     }
-    const float sc = PAIR ? scale * sigma : sigma;
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       float sn, cs;
-      sincospif(sc * v[e].x, &sn, &cs);
+      sincospif(atoms ? sigma * v[e].x : 0.f, &sn, &cs);
       v[e] = make_float2(cs, sn);
     }
     if (mode == 2) {
