@@ -7,14 +7,16 @@
 // psi~ itself (one process's share of a frame-sharded transform).  The stack is read once and the
 // result written once; the dense forms of the transform read it two or three times, write a
 // residual or split operands and do O(F) work per element where this does O(log F).  1024 frames x
-// 65536 q: 14.6 ms dense FP32, 0.23 ms here (3.5 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
-// 0.17 ms.  Bound by latency: no pipe is above half of its rate (shared memory 48%, FP32 47%, DRAM 42% in
-// the image at 256 frames; 51% of the issue slots by the 8 warps that fit in the chirp-z form at 1024).
+// 65536 q: 14.6 ms dense FP32, 0.27 ms here (3.0 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
+// 0.17 ms.  Bound by latency and the FP32 pipe.
 //
-// Mean: every frame is first referred to the column's first frame, r1_n = psi_n - psi_0, which
-// rounds at the scale of the fluctuation (the difference of two nearly equal floats is exact), then
-// the mean of r1 is subtracted.  What the large static part could cost in precision is gone in the
-// first step, so both sums are plain FP32; columns that do not change give exactly zero.
+// Mean and residual to FP64-class precision, as the dense forms have them: a column is summed as FP32
+// pairs (error-free two-sums, in the thread, over the lanes and over the warps), divided by F as a pair, and
+// r_n = psi_n - mean is formed exactly before it is rounded, once.  Columns that do not change give exactly
+// zero.  Plain FP32 sums of psi_n - psi_0 are faster (1024 frames x 65536 q 235 us, 266 now; image of 32
+// probes at 256 frames 435, 521; 501 frames 315, 346), but their error, the same in every frame, came
+// back F-fold in bin 0: up to 15 times the rounding of the sum itself in columns whose first frame stands
+// out.
 //
 // Frame counts: the engine's own lengths directly; any other F up to 2048 by Bluestein's chirp-z
 // identity m n = (m^2 + n^2 - (m - n)^2) / 2, as a cyclic convolution of length M >= 2 F - 1 with a
@@ -34,11 +36,13 @@ enum TimeOut { TIME_S, TIME_DETECTOR, TIME_TILDE };
 
 // Shape of a kernel: elements per thread, columns per CTA, CTAs per SM, and whether a thread loads its
 // next column while it transforms this one.  Per length the fastest of 4 to 14 shapes on one GB300
-// (ps per element of the stack; one shape for all uses -> these): 256 points S 3.21 -> 2.95, image
-// 3.05 -> 2.85, chirp-z 7.64 -> 7.08; 512: S 4.99 -> 3.39, image 4.88 -> 3.14, chirp-z 11.4 -> 8.0;
-// 1024: S 7.02 -> 4.95, image 5.41 -> 4.42, chirp-z 13.0 -> 11.2; 2048: S 7.91 -> 7.54, image 7.43 ->
-// 5.87, chirp-z 19.8 -> 14.9; 4096: chirp-z 27.7 -> 16.9.  16 columns are whole 128-byte lines of the
-// stack; more columns of the long transforms would leave one CTA per SM.
+// (ps per element of the stack; one shape for all uses -> these, before the mean was summed in pairs): 256
+// points S 3.21 -> 2.95, image 3.05 -> 2.85, chirp-z 7.64 -> 7.08; 512: S 4.99 -> 3.39, image 4.88 -> 3.14,
+// chirp-z 11.4 -> 8.0; 1024: S 7.02 -> 4.95, image 5.41 -> 4.42, chirp-z 13.0 -> 11.2; 2048: S 7.91 -> 7.54,
+// image 7.43 -> 5.87, chirp-z 19.8 -> 14.9; 4096: chirp-z 27.7 -> 16.9.  Now S, image, chirp-z S at 256 points
+// 3.05, 3.07, 7.18; 512: 3.79, 3.14, 8.52; 1024: 4.97, 4.38, 11.3; 2048: 7.53, 5.71, 14.8; two CTAs an SM of
+// 256 points in the image, 3.38, or six of half the columns, 3.19, lose to three.  16 columns are whole
+// 128-byte lines of the stack; more columns of the long transforms would leave one CTA per SM.
 struct TimeShape {
   int e, c, minb;
   bool prefetch;
@@ -129,11 +133,44 @@ __device__ __forceinline__ void column_pairs(float* hi, float* lo, int c, int& e
   }
 }
 
+// Complex FP32 pairs, both parts in packed instructions.
+__device__ __forceinline__ float2 shfl_xor2(float2 a, int o) {
+  return make_float2(__shfl_xor_sync(0xffffffffu, a.x, o), __shfl_xor_sync(0xffffffffu, a.y, o));
+}
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = a + b;
+  const float2 bb = s - a;
+  e = (a - (s - bb)) + (b - bb);
+}
+// (h, l) += (xh, xl)
+__device__ __forceinline__ void pair_add2(float2& h, float2& l, float2 xh, float2 xl) {
+  float2 e;
+  two_sum2(h, xh, h, e);
+  l = (l + xl) + e;
+}
+// (h + l) / F as (mh, ml): mh is the rounded product with 1 / F, whose remainder h - F mh is exact
+// (a few F units of mh's last place), and ml the quotient of what is left, corrected once, so that a
+// column of F equal frames has exactly that mean.
+__device__ __forceinline__ void pair_div2(float2 h, float2 l, float F, float inv, float2& mh, float2& ml) {
+  mh = inv * h;
+  const float2 rem = fma2(-F, mh, h) + l;
+  const float2 q = inv * rem;
+  ml = fma2(inv, fma2(-F, q, rem), q);
+}
+// x - (mh + ml), the first difference exact, so rounded once at the scale of the result
+__device__ __forceinline__ float2 pair_sub2(float2 x, float2 mh, float2 ml) {
+  float2 s, e;
+  two_sum2(x, make_float2(-mh.x, -mh.y), s, e);
+  return s + (e - ml);
+}
+
 template <int N, int OUT, bool BLUE>
-__global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT, BLUE>::MINB) k_time_fft(const TimeArgs a) {
+__global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT, BLUE>::MINB)
+    k_time_fft(const TimeArgs a) {
   grid_dependency_wait();
   using TC = TimeCfg<N, OUT, BLUE>;
   constexpr int E = TC::E, T = TC::T, C = TC::C, WARPS = TC::THREADS / 32;
+  constexpr int IN = BLUE ? E / 2 : E;  // chirp-z: N >= 2 F - 1 is even, so t + T e < F only for e < E / 2
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int64_t p = blockIdx.y + (int64_t)gridDim.y * blockIdx.z;
@@ -149,7 +186,7 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
     for (int e = 0; e < E; ++e) hi[e] = lo[e] = 0.f;
   }
   const int64_t tile0 = (int64_t)blockIdx.x * a.tpc, tile1 = tile0 + a.tpc < ntiles ? tile0 + a.tpc : ntiles;
-  // frames t + T e of column tile * C + c, and what every frame is referred to
+  // frames t + T e of column tile * C + c (zeros past the last one); x0: the static reference (TIME_TILDE)
   const auto load = [&](float2 (&u)[E], float2& x0, int64_t tile) {
     const int64_t j = tile * C + c, jj = j < a.nsel ? j : a.nsel - 1;  // past the end: the last one, unstored
     const int64_t q = a.in_qsel ? a.in_qsel[jj] : jj;
@@ -163,11 +200,10 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
       }
     } else {
       const float2* col = a.psi + (size_t)p * F * a.in_nq + q;
-      x0 = col[0];
 #pragma unroll
       for (int e = 0; e < E; ++e) {
         const int n = t + T * e;
-        u[e] = !BLUE || n < F ? col[(size_t)n * a.in_nq] : x0;
+        u[e] = !BLUE || n < F ? col[(size_t)n * a.in_nq] : make_float2(0.f, 0.f);
       }
     }
   };
@@ -178,7 +214,7 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
     const int64_t q = a.in_qsel ? a.in_qsel[jj] : jj;
     const bool part = OUT == TIME_TILDE;
     const float2* col = a.psi + (size_t)p * (part ? a.nf : (int64_t)F) * a.in_nq + q;
-    x0 = part ? a.ref[(size_t)p * a.in_nq + q] : col[0];
+    if (part) x0 = a.ref[(size_t)p * a.in_nq + q];
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       const int64_t n = t + T * e - (part ? a.f0 : 0);
@@ -193,16 +229,16 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
     for (int e = 0; e < E; ++e) {
       const int64_t n = t + T * e - (OUT == TIME_TILDE ? a.f0 : 0);
       const bool in = OUT == TIME_TILDE ? n >= 0 && n < a.nf : !BLUE || n < F;
-      u[e] = in ? slots[TC::THREADS * e] : x0;
+      u[e] = in ? slots[TC::THREADS * e] : OUT == TIME_TILDE ? x0 : make_float2(0.f, 0.f);
     }
   };
-  float2 v[E], x0;
+  float2 v[E], x0 = make_float2(0.f, 0.f);
   if (TC::ASYNC) fetch(x0, tile0);
   else load(v, x0, tile0);
   for (int64_t tile = tile0; tile < tile1; ++tile) {
     const int64_t j = tile * C + c;
     const bool live = j < a.nsel;
-    float2 next[E], next0;
+    float2 next[E], next0 = x0;
     if (TC::ASYNC) collect(v, x0);
     if (TC::PREFETCH && tile + 1 < tile1) load(next, next0, tile + 1);
     if constexpr (OUT == TIME_TILDE) {
@@ -210,28 +246,40 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
       for (int e = 0; e < E; ++e) v[e] = v[e] - x0;
       if (TC::ASYNC) __syncthreads();  // every slot has been read
     } else {
-      float2 sum = make_float2(0.f, 0.f);
+      float2 hs = v[0], ls = make_float2(0.f, 0.f);
 #pragma unroll
-      for (int e = 0; e < E; ++e) {
-        v[e] = v[e] - x0;
-        sum = sum + v[e];
+      for (int e = 1; e < IN; ++e) {
+        float2 err;
+        two_sum2(hs, v[e], hs, err);
+        ls = ls + err;
       }
       // the column's sum: over the lanes of a warp that share it, then over the warps
 #pragma unroll
-      for (int o = C; o < 32; o <<= 1) {
-        sum.x += __shfl_xor_sync(0xffffffffu, sum.x, o);
-        sum.y += __shfl_xor_sync(0xffffffffu, sum.y, o);
-      }
+      for (int o = C; o < 32; o <<= 1)
+        pair_add2(hs, ls, shfl_xor2(hs, o), shfl_xor2(ls, o));
+      float4* part = reinterpret_cast<float4*>(smraw);  // [WARPS][C]
       __syncthreads();  // the previous tile's readers of the scratch are done
-      if ((threadIdx.x & 31) < C) sm[(threadIdx.x >> 5) * C + c] = sum;
+      if ((threadIdx.x & 31) < C) part[(threadIdx.x >> 5) * C + c] = make_float4(hs.x, hs.y, ls.x, ls.y);
       __syncthreads();
-      sum = make_float2(0.f, 0.f);
+      // the lanes of a column share the warps' sums, then add theirs
+      constexpr int L = 32 / C < WARPS ? 32 / C : WARPS;
+      static_assert(WARPS % L == 0, "every lane takes as many of the warps' sums");
+      const int l0 = (threadIdx.x & 31) / C % L;
+      float4 q = part[l0 * C + c];
+      hs = make_float2(q.x, q.y);
+      ls = make_float2(q.z, q.w);
 #pragma unroll
-      for (int w = 0; w < WARPS; ++w) sum = sum + sm[w * C + c];
-      const float inv = 1.f / (float)F;
-      const float2 mean = make_float2(sum.x * inv, sum.y * inv);
+      for (int w = L; w < WARPS; w += L) {
+        q = part[(w + l0) * C + c];
+        pair_add2(hs, ls, make_float2(q.x, q.y), make_float2(q.z, q.w));
+      }
 #pragma unroll
-      for (int e = 0; e < E; ++e) v[e] = !BLUE || t + T * e < F ? v[e] - mean : make_float2(0.f, 0.f);
+      for (int o = C; o < C * L; o <<= 1) pair_add2(hs, ls, shfl_xor2(hs, o), shfl_xor2(ls, o));
+      float2 mh, ml;
+      pair_div2(hs, ls, (float)F, 1.f / (float)F, mh, ml);
+#pragma unroll
+      for (int e = 0; e < E; ++e)
+        v[e] = e < IN && (!BLUE || t + T * e < F) ? pair_sub2(v[e], mh, ml) : make_float2(0.f, 0.f);
     }
     // (both branches have passed a barrier after the slots were read)
     if (TC::ASYNC && tile + 1 < tile1) fetch(x0, tile + 1);
