@@ -36,7 +36,7 @@ def _newest_input():
 
 def build(force: bool = False, verbose: bool = False, extra=()) -> str:
     """Build (or reuse) libtacaw.so; returns its path.  TACAW_NVCC_DEFINES (space-separated
-    -D flags) selects tuning variants of the kernels, e.g. "-DTACAW_FFT_MINB=2"."""
+    -D flags) selects tuning variants of the kernels, e.g. "-DTACAW_TUNE_FORCE=2"."""
     defines = os.environ.get("TACAW_NVCC_DEFINES", "").split()
     stamp = LIB + ".defines"
     same = os.path.exists(stamp) and open(stamp).read() == " ".join(defines)

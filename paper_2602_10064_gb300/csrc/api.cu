@@ -302,7 +302,8 @@ int check_params(tacaw_ctx* ctx, const tacaw_params* p) {
     return set_err(ctx, TACAW_EINVAL,
                    "grid %dx%d: nx, ny must be powers of two in [32, 1024] or one of 96, 192, 384, 768, 1152",
                    p->nx, p->ny);
-  if (p->n_slices < 1 || p->n_slices > 256) return set_err(ctx, TACAW_EINVAL, "n_slices %d not in [1, 256]", p->n_slices);
+  if (p->n_slices < 1 || p->n_slices > 256)
+    return set_err(ctx, TACAW_EINVAL, "n_slices %d not in [1, 256]", p->n_slices);
   for (int i = 0; i < 3; ++i)
     if (!(p->cell[i] > 0.0) || !std::isfinite(p->cell[i])) return set_err(ctx, TACAW_EINVAL, "cell[%d] must be > 0", i);
   if (!(p->voltage_ev > 0.0)) return set_err(ctx, TACAW_EINVAL, "voltage_ev must be > 0");
@@ -664,7 +665,8 @@ int make_slots(tacaw_ctx* ctx, const int32_t* Z, int64_t A, bool z_on_device, bo
     int s = -1;
     for (size_t i = 0; i < ctx->ffZ.size(); ++i)
       if (ctx->ffZ[i] == Z[j]) s = (int)i;
-    if (s < 0) return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, Z[j]);
+    if (s < 0)
+      return set_err(ctx, TACAW_EINVAL, "atom %lld has Z=%d, not in the form-factor table", (long long)j, Z[j]);
     hs[j] = (int8_t)s;
   }
   CK(sc.get(d_slot, A));
@@ -836,8 +838,10 @@ int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const 
                fy = 5.0 * p.ny * std::log2((double)p.ny);
   if (!bl) {
     if (pp) {
-      ProfScope ps(ctx, "row_pot_t", sc.st, (double)pp->planes * p.ny * W8 + row * 8.0 * p.nx, (double)pp->planes * p.ny * fx);
-      CK(launch_row_pot_out(geo, g->band, pp->Ap, pp->planes, pp->sp, 2, sig, nullptr, t, (int)ctx->static_band, sc.st));
+      ProfScope ps(ctx, "row_pot_t", sc.st, (double)pp->planes * p.ny * W8 + row * 8.0 * p.nx,
+                   (double)pp->planes * p.ny * fx);
+      CK(launch_row_pot_out(geo, g->band, pp->Ap, pp->planes, pp->sp, 2, sig, nullptr, t, (int)ctx->static_band,
+                            sc.st));
     } else {
       ProfScope ps(ctx, "row_vt", sc.st, row * 12.0 * p.nx, 0);
       CK(launch_row_vt(geo, g->band, V, nfs, 0, sig, t, sc.st));
@@ -847,7 +851,8 @@ int transmission_from(tacaw_ctx* ctx, const tacaw_params& p, GeoCache* g, const 
   float2* Bt = tb.Bt;
   float2* At = compact ? t : tb.At;
   if (pp) {
-    ProfScope ps(ctx, "row_pot_t", sc.st, ((double)pp->planes * p.ny + row) * W8, ((double)pp->planes * p.ny + row) * fx);
+    ProfScope ps(ctx, "row_pot_t", sc.st, ((double)pp->planes * p.ny + row) * W8,
+                 ((double)pp->planes * p.ny + row) * fx);
     CK(launch_row_pot_out(geo, g->band, pp->Ap, pp->planes, pp->sp, 1, sig, nullptr, Bt, (int)ctx->static_band, sc.st));
   } else {
     ProfScope ps(ctx, "row_vt", sc.st, row * (4.0 * p.nx + W8), row * fx);
@@ -909,7 +914,8 @@ int build_probes(tacaw_ctx* ctx, const tacaw_params& p, const tacaw_probe& pr, S
     CK(launch_probe_col(geo, ap, d_ex, d_ey, d_chi, P, (float)(1.0 / std::sqrt((double)count)), Bpr, sc.st));
   }
   {
-    ProfScope ps(ctx, "probe_row", sc.st, (double)P * ny * (Wp + nx) * 8, (double)P * ny * 5.0 * nx * std::log2((double)nx));
+    ProfScope ps(ctx, "probe_row", sc.st, (double)P * ny * (Wp + nx) * 8,
+                 (double)P * ny * 5.0 * nx * std::log2((double)nx));
     CK(launch_probe_row(geo, ap, Bpr, P, (float)(1.0 / std::sqrt((double)nx * ny)), *psi0, sc.st));
   }
   return TACAW_OK;
@@ -1092,7 +1098,8 @@ uint64_t run_footprint(tacaw_ctx* ctx, const tacaw_params& p, int P, int64_t Fr,
   const double chunk = (double)pl.rt.chunk, sb = pl.rt.sb, Pb = pl.Pb;
   const double tsz = (pl.tf ? plane : nq) * 8;
   double b = 0;
-  b += (double)F * A * (12 + 16 + 16 + 1) + (double)F * (S + 1) * 4 + A;  // positions, records (binned, row-sorted), slices, slots
+  // positions, records (binned, row-sorted), slices, slots
+  b += (double)F * A * (12 + 16 + 16 + 1) + (double)F * (S + 1) * 4 + A;
   b += (double)F * S * (p.ny / SPREAD_YB + 1) * 4;                      // row-block offsets
   b += chunk * sb * plane * 8 * (g->npair + 2);                         // Bp, Ap, Bt
   if (!pl.tf) b += chunk * sb * plane * 8;                              // At
@@ -1190,7 +1197,8 @@ int tacaw_bin_slices(tacaw_ctx* ctx, const tacaw_params* params, const float* po
   TRY_RC(check_params(ctx, params));
   if (n_atoms < 0 || nf < 1) return set_err(ctx, TACAW_EINVAL, "n_atoms >= 0 and nf >= 1 required");
   if (n_atoms == 0) return TACAW_OK;
-  if (!is_device_ptr(pos) || !is_device_ptr(slice_out)) return set_err(ctx, TACAW_EINVAL, "pos, slice_out must be device pointers");
+  if (!is_device_ptr(pos) || !is_device_ptr(slice_out))
+    return set_err(ctx, TACAW_EINVAL, "pos, slice_out must be device pointers");
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
   CK(launch_slice_index(pos, nf * n_atoms, bin_geom(params->cell[0], params->cell[1], params->cell[2], params->nx,
@@ -1271,7 +1279,8 @@ int tacaw_propagate(tacaw_ctx* ctx, const tacaw_params* params, const float* V, 
   if (pr.alpha_mrad <= 0.0 && !pr.psi0 && pr.n_probes != 1)
     return set_err(ctx, TACAW_EINVAL, "a plane wave takes exactly one probe");
   if (pr.psi0 && !is_device_ptr(pr.psi0)) return set_err(ctx, TACAW_EINVAL, "probe psi0 must be a device pointer");
-  if (!is_device_ptr(V) || !is_device_ptr(psi_k_out)) return set_err(ctx, TACAW_EINVAL, "V, psi_k_out must be device pointers");
+  if (!is_device_ptr(V) || !is_device_ptr(psi_k_out))
+    return set_err(ctx, TACAW_EINVAL, "V, psi_k_out must be device pointers");
   CK(cudaSetDevice(ctx->device));
   cudaStream_t st = (cudaStream_t)stream;
   GeoCache* g;

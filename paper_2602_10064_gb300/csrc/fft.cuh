@@ -295,13 +295,13 @@ __device__ __forceinline__ void dft_r(float2* u) {
 // Lengths 3 * 2^k (96 .. 768) and 9 * 2^7 (1152) besides the powers of two.
 __host__ __device__ constexpr bool fft_pow2(int n) { return n > 0 && (n & (n - 1)) == 0; }
 
-// Elements per thread (E) for a transform of length N: 8 or 16 for powers of two (8 for
-// N <= 64), 24 for the lengths with a factor 3: two passes for 96 and 192, three for the others
-// (8 x 8 x 12 beats 24 x 4 x 8 for 768 by 10%, but 8 x 12 x 12 loses to 24 x 6 x 8 for 1152 by 10%).  A kernel picks E per pass direction (powers of two); T = N / E threads share one
-// transform.
-template <int N, int EPREF>
+// Elements per thread (E) for a transform of length N: 16 for powers of two (8 for N <= 64), 24 for
+// the lengths with a factor 3: two passes for 96 and 192, three for the others (8 x 8 x 12 beats
+// 24 x 4 x 8 for 768 by 10%, but 8 x 12 x 12 loses to 24 x 6 x 8 for 1152 by 10%).  T = N / E threads
+// share one transform.
+template <int N>
 struct FftPlan {
-  static constexpr int E = fft_pow2(N) ? ((N <= 64) ? 8 : EPREF) : 24;
+  static constexpr int E = fft_pow2(N) ? (N <= 64 ? 8 : 16) : 24;
   static constexpr int T = N / E;
 };
 
@@ -415,9 +415,7 @@ __device__ __forceinline__ void fft_pass(float2 (&v)[E], float2* sm, const Idx& 
 // SIGN = -1 forward, +1 inverse.  All T threads of the group call it together; sm (through
 // idx) is the group's private scratch; sync is the barrier of the threads sharing it.  tw
 // points at the context's pass tables.
-// PLAN selects the radix schedule where there is a choice: 0 = radix-16 passes, 1 = radix-8
-// passes (two butterflies per thread and pass) for 512 and 1024 points with E = 16.
-template <int N, int SIGN, int PLAN = 0, int E, class Idx, class Sync>
+template <int N, int SIGN, int E, class Idx, class Sync>
 __device__ __forceinline__ void fft(float2 (&v)[E], float2* sm, const Idx& idx, int t,
                                     const float2* __restrict__ tw, const Sync& sync) {
   if constexpr (N == 32) {
@@ -438,37 +436,12 @@ __device__ __forceinline__ void fft(float2 (&v)[E], float2* sm, const Idx& idx, 
   } else if constexpr (E == 32 && N == 1024) {
     fft_pass<1024, E, 32, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<1024, E, 32, 32, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 8 && N == 128) {
-    fft_pass<128, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<128, E, 4, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<128, E, 4, 32, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 8 && N == 256) {
-    fft_pass<256, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<256, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<256, E, 4, 64, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 8 && N == 512) {
-    fft_pass<512, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<512, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<512, E, 8, 64, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (E == 8 && N == 1024) {
-    fft_pass<1024, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<1024, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<1024, E, 4, 64, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<1024, E, 4, 256, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (N == 128) {
     fft_pass<128, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<128, E, 8, 16, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (N == 256) {
     fft_pass<256, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<256, E, 16, 16, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (PLAN == 1 && N == 512) {
-    fft_pass<512, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<512, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<512, E, 8, 64, SIGN, true>(v, sm, idx, t, tw, sync);
-  } else if constexpr (PLAN == 1 && N == 1024) {
-    fft_pass<1024, E, 8, 1, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<1024, E, 8, 8, SIGN, false>(v, sm, idx, t, tw, sync);
-    fft_pass<1024, E, 16, 64, SIGN, true>(v, sm, idx, t, tw, sync);
   } else if constexpr (N == 512) {
     fft_pass<512, E, 16, 1, SIGN, false>(v, sm, idx, t, tw, sync);
     fft_pass<512, E, 16, 16, SIGN, false>(v, sm, idx, t, tw, sync);

@@ -21,12 +21,11 @@ namespace tacaw {
 
 // Per-kernel variants of the FFT pass kernels, chosen per transform length by the autotuner
 // (paper_2602_10064_gb300/tune.py), which times every variant on GB300 and writes
-// tuning_table.h.  Variant bits: 1 = radix-8 plans (512 and 1024 points, 16 elements per
-// thread), 2 = 1.5 to 2 times as many resident threads per SM (fewer registers each), 4 = column
-// passes only: twice the columns per CTA, so that each load instruction covers whole 128-byte
-// lines, 8 = 32 elements per thread for the powers of two from 128 points (two-pass
-// transforms, about 170 registers).  TACAW_TUNE_FORCE=v builds every kernel as variant v (the
-// tuner's measurement builds).
+// tuning_table.h.  Variant bits: 2 = 1.5 to 2 times as many resident threads per SM (fewer
+// registers each), 4 = column passes only: twice the columns per CTA, so that each load
+// instruction covers whole 128-byte lines, 8 = 32 elements per thread for the powers of two from
+// 128 points (two-pass transforms, about 170 registers).  TACAW_TUNE_FORCE=v builds every kernel
+// as variant v (the tuner's measurement builds).
 enum KernelId {
   K_SPLAT_ROW, K_COL_POT, K_ROW_POT_OUT, K_ROW_VT, K_COL_T, K_ROW_TOUT, K_PROBE_COL, K_PROBE_ROW,
   K_SLICE_ROW, K_SLICE_COL, K_SLICE_ROW_SCAN
@@ -42,7 +41,6 @@ struct Tuned {
   static constexpr int V = TACAW_TUNE_FORCE >= 0 ? TACAW_TUNE_FORCE : tuned_variant(K, N);
   static constexpr bool COLUMN = K == K_COL_POT || K == K_COL_T || K == K_PROBE_COL || K == K_SLICE_COL;
   static constexpr int EV = (V & 8) ? 1 : 0;
-  static constexpr int PLAN = (V & 1) && !EV;
   static constexpr int WIDE = (COLUMN && (V & 4)) ? 1 : 0;
   // resident CTAs per SM requested for a CTA of `threads`: `target` threads per SM; variant & 2: 1.5
   // times as many, or twice where that makes no difference to the CTAs and in the spreading pass
@@ -52,14 +50,6 @@ struct Tuned {
     return n > 1 ? n : 1;
   }
 };
-
-// Elements per thread of the row and of the column transforms (8 or 16).
-#ifndef TACAW_ROW_E
-#define TACAW_ROW_E 16
-#endif
-#ifndef TACAW_COL_E
-#define TACAW_COL_E 16
-#endif
 
 // Largest power of two <= x (x >= 1).
 __host__ __device__ constexpr int floor_pow2(int x) {
@@ -80,7 +70,7 @@ __host__ __device__ constexpr int floor_pow2(int x) {
 // synchronise several warps (768 points 4.33, 4.43; 1152 points 4.81, 4.90).
 template <int N, int EV = 0, int SMALL = 64, int LARGE = 192>
 struct RowCfg {
-  static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N, TACAW_ROW_E>::E;
+  static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N>::E;
   static constexpr int T = N / E;
   static constexpr int TARGET = E >= 24 ? 384 : 512;
   static constexpr int G0 = (E < 24 ? SMALL : T < 32 ? LARGE : 192) / T;
@@ -94,7 +84,7 @@ struct RowCfg {
 // 128 points 3.23 -> 2.97 ps a point in the slice pass; 256 points lose 5% with 8 columns.
 template <int N, int WIDE = 0, int EV = 0>
 struct ColCfg {
-  static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N, TACAW_COL_E>::E;
+  static constexpr int E = (EV && fft_pow2(N) && N >= 128) ? 32 : FftPlan<N>::E;
   static constexpr int T = N / E;
   static constexpr int TARGET = E >= 24 ? 384 : 512;
   static constexpr int FULL = TARGET / 2 / T, HALF = TARGET / 4 / T;
@@ -136,7 +126,7 @@ __device__ __forceinline__ auto group_sync(int g) {
 }
 
 // CTAs of a column pass: the in-band columns c < W only, C per CTA.  The padding columns up to Wp
-// are never read by a row pass (band_x_col maps no x to them), so they need no transform.
+// are never read by a row pass (no x maps to them), so they need no transform.
 static int col_blocks(const Band& b, int C) { return (b.W + C - 1) / C; }
 
 // Batch index over (grid.y, grid.z); batches beyond nb return before any barrier.
@@ -439,7 +429,8 @@ cudaError_t launch_sort_rows(const AtomRec* recs, const int* offs, int64_t A, in
     const cudaError_t e = cudaFuncSetAttribute(k_sort_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
   }
-  return launch_after(k_sort_rows, (unsigned)((nseg + SORT_WARPS - 1) / SORT_WARPS), SORT_WARPS * 32, smem, st,  recs, offs, (int)A, S, (int)nseg, ny, out, boffs);
+  return launch_after(k_sort_rows, (unsigned)((nseg + SORT_WARPS - 1) / SORT_WARPS), SORT_WARPS * 32, smem, st, recs,
+                      offs, (int)A, S, (int)nseg, ny, out, boffs);
 }
 
 cudaError_t launch_slice_index(const float* pos, int64_t n, const BinGeom& g, int* slice_out, cudaStream_t st) {
@@ -452,7 +443,9 @@ cudaError_t launch_bin(const float* pos, int64_t A, int64_t nf, const BinGeom& g
                        AtomRec* rec, uint8_t* key, AtomRec* recs, int* offs, cudaStream_t st) {
   if (g.S > BIN_MAX_S || nf <= 0) return cudaErrorInvalidValue;
   cudaError_t e = cudaSuccess;
-  if (A > 0) e = launch_after(k_atoms, batch_grid((int)((A + 255) / 256), nf), 256, 0, st, pos, (int)A, nf, g, slot_of_atom, rec, key);
+  if (A > 0)
+    e = launch_after(k_atoms, batch_grid((int)((A + 255) / 256), nf), 256, 0, st, pos, (int)A, nf, g, slot_of_atom, rec,
+                     key);
   if (e != cudaSuccess) return e;
   return launch_after(k_bin, (unsigned)nf, BIN_THREADS, 0, st, rec, key, (int)A, g.S, recs, offs);
 }
@@ -494,7 +487,6 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
                 int s0, int sb, int npair, int two, int nbatch, float beta, float2* __restrict__ Bp) {
   grid_dependency_wait();
   constexpr int E = SplatCfg<NX>::E, T = SplatCfg<NX>::T, G = SplatCfg<NX>::G, NT = SplatCfg<NX>::THREADS;
-  constexpr int PL = Tuned<K_SPLAT_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);                     // FFT scratch (after spreading)
   float2* acc = reinterpret_cast<float2*>(smraw);                    // [G][NX]
@@ -548,7 +540,6 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
       n1 = bo[b_hi + 1] - s1;
     }
     const int M = n1 + n2;
-
 
     for (int base = 0; base < M; base += NT) {
       // 1. the batch's candidate records (atoms of other species pairs are marked and skipped)
@@ -609,7 +600,8 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
         }
         if (wyc == 0.f) continue;
         const int d = wrap3<NX>(x0 - t + NX);
-        for (int off = (T - d % T) % T; off < W2; off += T) arow[2 * wrap3<NX>(x0 + off) + im] += wyc * phx[c * W2 + off];
+        for (int off = (T - d % T) % T; off < W2; off += T)
+          arow[2 * wrap3<NX>(x0 + off) + im] += wyc * phx[c * W2 + off];
       }
       __syncthreads();
     }
@@ -618,7 +610,7 @@ __global__ void __launch_bounds__(SplatCfg<NX>::THREADS, minb_of<K_SPLAT_ROW, NX
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = acc[g * NX + t + T * e];
   __syncthreads();  // the FFT scratch of one group overlaps the accumulators of the next
-  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
+  fft<NX, -1>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   store_row<NX, MB>(v, Bp + ((size_t)bidx * ny + y0 + g) * b.Wp, b, t);
 }
@@ -631,7 +623,6 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
   grid_dependency_wait();
   using CC = ColPotCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
-  constexpr int PL = Tuned<K_COL_POT, NY>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int fs = batch_index();
@@ -647,11 +638,11 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
     float2 v[E];
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = src[(size_t)(t + T * e) * Wp];
-    fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+    fft<NY, -1>(v, sm, idx, t, tw, sync);
     const float2* m = mtab + cc;
 #pragma unroll
     for (int e = 0; e < E; ++e) v[e] = cmul(m[(size_t)(t + T * e) * Wp], v[e]);
-    fft<NY, +1, PL>(v, sm, idx, t, tw, sync);
+    fft<NY, +1>(v, sm, idx, t, tw, sync);
     float2* dst = Ap + (size_t)fs * NY * Wp + cc;
 #pragma unroll
     for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = v[e];
@@ -664,12 +655,12 @@ __global__ void __launch_bounds__(ColPotCfg<NY>::THREADS, minb_of<K_COL_POT, NY,
       float2 v[E];
 #pragma unroll
       for (int e = 0; e < E; ++e) v[e] = src[(size_t)(t + T * e) * Wp];
-      fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+      fft<NY, -1>(v, sm, idx, t, tw, sync);
       const float2* m = mtab + (size_t)pr * NY * Wp + cc;
 #pragma unroll
       for (int e = 0; e < E; ++e) acc[e] = acc[e] + cmul(m[(size_t)(t + T * e) * Wp], v[e]);
     }
-    fft<NY, +1, PL>(acc, sm, idx, t, tw, sync);
+    fft<NY, +1>(acc, sm, idx, t, tw, sync);
     float2* dst = Ap + (size_t)fs * NY * Wp + cc;
 #pragma unroll
     for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = acc[e];
@@ -693,7 +684,6 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
                   float* __restrict__ V, float2* __restrict__ out) {
   grid_dependency_wait();
   constexpr int E = PotOutCfg<NX>::E, T = PotOutCfg<NX>::T, G = PotOutCfg<NX>::G;
-  constexpr int PL = Tuned<K_ROW_POT_OUT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int bi = batch_index();
@@ -703,7 +693,7 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
   const auto sync = group_sync<T>(g);
   float2 v[E];
   load_row<NX, MB>(v, Ap + ((size_t)bi * ny + y) * b.Wp, b, t);
-  fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
+  fft<NX, +1>(v, sm, idx, t, geo.tw, sync);
   // slices [s, s_end) of frame f come from this plane, s - s_first its part
   int f = 0, s_first = 0, s = 0, s_end = 1;
   if (PAIR) {
@@ -744,7 +734,7 @@ __global__ void __launch_bounds__(PotOutCfg<NX>::THREADS, minb_of<K_ROW_POT_OUT,
       for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
       continue;
     }
-    fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
+    fft<NX, -1>(v, sm, idx, t, geo.tw, sync);
     store_row<NX, MB>(v, out + (plane * ny + y) * b.Wp, b, t);
   }
 }
@@ -758,7 +748,6 @@ __global__ void __launch_bounds__(RowVtCfg<NX>::THREADS, minb_of<K_ROW_VT, NX, R
              float2* __restrict__ out) {
   grid_dependency_wait();
   constexpr int E = RowVtCfg<NX>::E, T = RowVtCfg<NX>::T, G = RowVtCfg<NX>::G;
-  constexpr int PL = Tuned<K_ROW_VT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int fs = batch_index();
@@ -777,7 +766,7 @@ __global__ void __launch_bounds__(RowVtCfg<NX>::THREADS, minb_of<K_ROW_VT, NX, R
     for (int e = 0; e < E; ++e) out[row + t + T * e] = v[e];
     return;
   }
-  fft<NX, -1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
+  fft<NX, -1>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   store_row_compact<NX>(v, out + ((size_t)fs * ny + y) * b.Wp, b, t);
 }
@@ -789,7 +778,6 @@ __global__ void __launch_bounds__(ColTCfg<NY>::THREADS, minb_of<K_COL_T, NY, Col
   grid_dependency_wait();
   using CC = ColTCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
-  constexpr int PL = Tuned<K_COL_T, NY>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int fs = batch_index();
@@ -803,14 +791,14 @@ __global__ void __launch_bounds__(ColTCfg<NY>::THREADS, minb_of<K_COL_T, NY, Col
   float2 v[E];
 #pragma unroll
   for (int e = 0; e < E; ++e) v[e] = src[(size_t)(t + T * e) * Wp];
-  fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+  fft<NY, -1>(v, sm, idx, t, tw, sync);
   const int nb = cc < b.W ? b.colnb[cc] : -1;
 #pragma unroll
   for (int e = 0; e < E; ++e) {
     const int n = fftfreq_index(t + T * e, NY);
     v[e] = (abs(n) <= nb) ? scale * v[e] : make_float2(0.f, 0.f);
   }
-  fft<NY, +1, PL>(v, sm, idx, t, tw, sync);
+  fft<NY, +1>(v, sm, idx, t, tw, sync);
   float2* dst = At + (size_t)fs * NY * Wp + cc;
 #pragma unroll
   for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = v[e];
@@ -822,7 +810,6 @@ __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, N
     k_row_tout(Geo geo, Band b, const float2* __restrict__ At, int nbatch, float2* __restrict__ tout) {
   grid_dependency_wait();
   constexpr int E = RowToutCfg<NX>::E, T = RowToutCfg<NX>::T, G = RowToutCfg<NX>::G;
-  constexpr int PL = Tuned<K_ROW_TOUT, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int fs = batch_index();
@@ -830,7 +817,7 @@ __global__ void __launch_bounds__(RowToutCfg<NX>::THREADS, minb_of<K_ROW_TOUT, N
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
   float2 v[E];
   load_row_compact<NX>(v, At + ((size_t)fs * ny + y) * b.Wp, b, t);
-  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
+  fft<NX, +1>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   float2* dst = tout + ((size_t)fs * ny + y) * NX;
 #pragma unroll
@@ -885,7 +872,8 @@ __global__ void __launch_bounds__(256) k_probe_tables(ProbeTables q, const doubl
 cudaError_t launch_probe_tables(const ProbeTables& q, const double* xy, const int* nb, float2* ex, float2* ey,
                                 float2* chi, cudaStream_t st) {
   const int64_t n = (int64_t)q.P * (q.Wp + q.ny) + (chi ? (int64_t)q.ny * q.Wp : 0);
-  return launch_after(k_probe_tables, (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st, q, xy, nb, ex, ey, chi);
+  return launch_after(k_probe_tables, (unsigned)std::min<int64_t>((n + 255) / 256, 152 * 8), 256, 0, st, q, xy, nb,
+                      ex, ey, chi);
 }
 
 template <int NY>
@@ -895,7 +883,6 @@ __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL,
   grid_dependency_wait();
   using CC = ProbeColCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
-  constexpr int PL = Tuned<K_PROBE_COL, NY>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int p = batch_index();
@@ -910,7 +897,7 @@ __global__ void __launch_bounds__(ProbeColCfg<NY>::THREADS, minb_of<K_PROBE_COL,
     v[e] = (abs(n) <= nb) ? amp * cmul(exv, ey[(size_t)p * NY + row]) : make_float2(0.f, 0.f);
     if (chi && abs(n) <= nb) v[e] = cmul(v[e], chi[(size_t)row * ap.Wp + cc]);
   }
-  fft<NY, +1, PL>(v, sm, ColIdx<C, CC::SH>{c}, t, geo.tw, BlockSync{});
+  fft<NY, +1>(v, sm, ColIdx<C, CC::SH>{c}, t, geo.tw, BlockSync{});
   float2* dst = Bpr + (size_t)p * NY * ap.Wp + cc;
 #pragma unroll
   for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * ap.Wp] = v[e];
@@ -921,7 +908,6 @@ __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW,
     k_probe_row(Geo geo, Band ap, const float2* __restrict__ Bpr, int P, float scale, float2* __restrict__ psi0) {
   grid_dependency_wait();
   constexpr int E = ProbeRowCfg<NX>::E, T = ProbeRowCfg<NX>::T, G = ProbeRowCfg<NX>::G;
-  constexpr int PL = Tuned<K_PROBE_ROW, NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int p = batch_index();
@@ -929,7 +915,7 @@ __global__ void __launch_bounds__(ProbeRowCfg<NX>::THREADS, minb_of<K_PROBE_ROW,
   const int g = threadIdx.x / T, t = threadIdx.x % T, y = blockIdx.x * G + g, ny = geo.ny;
   float2 v[E];
   load_row_compact<NX>(v, Bpr + ((size_t)p * ny + y) * ap.Wp, ap, t);
-  fft<NX, +1, PL>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
+  fft<NX, +1>(v, sm, RowIdx<NX, E>{g * row_smem_stride<NX, E>()}, t, geo.tw,
                   group_sync<T>(g));
   float2* dst = psi0 + ((size_t)p * ny + y) * NX;
 #pragma unroll
@@ -968,7 +954,6 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
   grid_dependency_wait();
   using RC = SliceRowCfg<NX, TF>;
   constexpr int E = RC::E, T = RC::T, G = RC::G;
-  constexpr int PL = Tuned<slice_row_id<TF>(), NX>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int bi = batch_index();
@@ -1012,7 +997,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
   if constexpr (TF) {
     load_row<NX, MB>(v, ttab + ((size_t)(fl * S + s) * ny + y) * b.Wp, b, t);
     load(next, p0);
-    fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
+    fft<NX, +1>(v, sm, idx, t, geo.tw, sync);
 #pragma unroll
     for (int e = 0; e < E; ++e) tst[t + T * e] = v[e];
 #pragma unroll
@@ -1029,7 +1014,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
   }
   for (int p = p0; p < p1; ++p) {
     if (!TF && !TREG && p + 1 < p1) load(next, p + 1);
-    if (!FIRST) fft<NX, +1, PL>(v, sm, idx, t, geo.tw, sync);
+    if (!FIRST) fft<NX, +1>(v, sm, idx, t, geo.tw, sync);
     if (!TF && !TREG) cp_async_wait_all();
 #pragma unroll
     for (int e = 0; e < E; ++e) {
@@ -1037,7 +1022,7 @@ __global__ void __launch_bounds__(SliceRowCfg<NX, TF>::THREADS, minb_of<slice_ro
       if (FIRST && PLANE) v[e] = plane_amp * tv;
       else v[e] = cmul(v[e], tv);
     }
-    fft<NX, -1, PL>(v, sm, idx, t, geo.tw, sync);
+    fft<NX, -1>(v, sm, idx, t, geo.tw, sync);
     store_row<NX, MB>(v, Bpsi + ((size_t)(p * nfc + fl) * ny + y) * b.Wp, b, t);
     if (TF) return;  // one probe
     if (!TREG) {
@@ -1067,7 +1052,6 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
   grid_dependency_wait();
   using CC = SliceColCfg<NY>;
   constexpr int E = CC::E, T = CC::T, C = CC::C;
-  constexpr int PL = Tuned<K_SLICE_COL, NY>::PLAN;
   extern __shared__ __align__(16) unsigned char smraw[];
   float2* sm = reinterpret_cast<float2*>(smraw);
   const int w0 = batch_index() * wpb, w1 = w0 + wpb < nwaves ? w0 + wpb : nwaves;
@@ -1097,7 +1081,7 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
   for (int w = w0; w < w1; ++w) {
     float2 next[E];
     if (LOOP && w + 1 < w1) load(next, w + 1);
-    fft<NY, -1, PL>(v, sm, idx, t, tw, sync);
+    fft<NY, -1>(v, sm, idx, t, tw, sync);
 #pragma unroll
     for (int e = 0; e < E; ++e) {
       if (LOOP) {
@@ -1108,7 +1092,7 @@ __global__ void __launch_bounds__(SliceColCfg<NY>::THREADS, minb_of<K_SLICE_COL,
       }
     }
     if (!LAST) {
-      fft<NY, +1, PL>(v, sm, idx, t, tw, sync);
+      fft<NY, +1>(v, sm, idx, t, tw, sync);
       float2* dst = Apsi + (size_t)w * NY * Wp + cc;
 #pragma unroll
       for (int e = 0; e < E; ++e) dst[(size_t)(t + T * e) * Wp] = v[e];
@@ -1233,12 +1217,14 @@ static cudaError_t splat_row_n(const Geo& g, const Band& b, const AtomRec* recs,
     if (std_band<NX>(b, static_band)) {
       cudaError_t e = prep(k_splat_row<NX, NX / 3>, smem);
       if (e != cudaSuccess) return e;
-      return launch_after(k_splat_row<NX, NX / 3>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb, beta, Bp);
+      return launch_after(k_splat_row<NX, NX / 3>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A,
+                          S, s0, sb, npair, two, nb, beta, Bp);
     }
   }
   cudaError_t e = prep(k_splat_row<NX>, smem);
   if (e != cudaSuccess) return e;
-  return launch_after(k_splat_row<NX>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A, S, s0, sb, npair, two, nb, beta, Bp);
+  return launch_after(k_splat_row<NX>, grid, SplatCfg<NX>::THREADS, smem, st, g, b, recs, boffs, (int)A, S, s0, sb,
+                      npair, two, nb, beta, Bp);
 }
 cudaError_t launch_splat_row(const Geo& g, const Band& b, const AtomRec* recs, const int* boffs, int64_t A, int S,
                              int s0, int sb, int nfs, int npair, int two, float beta, float2* Bp, int static_band,
@@ -1263,7 +1249,6 @@ static cudaError_t col_pot_n(const Geo& g, const Band& b, const float2* Bp, cons
         if ((e = prep(k_col_pot<NY, false, WP>, CC::SMEM)) != cudaSuccess) return e;
         return launch_after(k_col_pot<NY, false, WP>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
       }
-      return cudaGetLastError();
     }
   }
   if (npair == 1) {
@@ -1273,7 +1258,6 @@ static cudaError_t col_pot_n(const Geo& g, const Band& b, const float2* Bp, cons
     if ((e = prep(k_col_pot<NY, false>, CC::SMEM)) != cudaSuccess) return e;
     return launch_after(k_col_pot<NY, false>, grid, CC::THREADS, CC::SMEM, st, g, b, Bp, mtab, npair, nfs, Ap);
   }
-  return cudaGetLastError();
 }
 cudaError_t launch_col_pot(const Geo& g, const Band& b, const float2* Bp, const float2* mtab, int npair, int nfs,
                            float2* Ap, int static_band, cudaStream_t st) {
@@ -1287,7 +1271,8 @@ static cudaError_t row_pot_out_p(const Geo& g, const Band& b, const float2* Ap, 
   const dim3 grid = batch_grid(g.ny / RC::G, nb);
   if constexpr (std_band_built<NX>()) {
     if (std_band<NX>(b, static_band)) {
-      return launch_after(k_row_pot_out<NX, PAIR, NX / 3>, grid, RC::THREADS, RC::SMEM, st, g, b, Ap, nb, sp, mode, sigma, V, out);
+      return launch_after(k_row_pot_out<NX, PAIR, NX / 3>, grid, RC::THREADS, RC::SMEM, st, g, b, Ap, nb, sp, mode,
+                          sigma, V, out);
     }
   }
   return launch_after(k_row_pot_out<NX, PAIR>, grid, RC::THREADS, RC::SMEM, st, g, b, Ap, nb, sp, mode, sigma, V, out);
@@ -1306,7 +1291,8 @@ cudaError_t launch_row_pot_out(const Geo& g, const Band& b, const float2* Ap, in
 template <int NX>
 static cudaError_t row_vt_n(const Geo& g, const Band& b, const float* V, int nfs, int bl, float sigma, float2* out,
                             cudaStream_t st) {
-  return launch_after(k_row_vt<NX>, batch_grid(g.ny / RowVtCfg<NX>::G, nfs), RowVtCfg<NX>::THREADS, RowVtCfg<NX>::SMEM, st,  g, b, V, nfs, bl, sigma, out);
+  return launch_after(k_row_vt<NX>, batch_grid(g.ny / RowVtCfg<NX>::G, nfs), RowVtCfg<NX>::THREADS,
+                      RowVtCfg<NX>::SMEM, st, g, b, V, nfs, bl, sigma, out);
 }
 cudaError_t launch_row_vt(const Geo& g, const Band& b, const float* V, int nfs, int bandlimit, float sigma,
                           float2* out, cudaStream_t st) {
@@ -1322,12 +1308,14 @@ static cudaError_t col_t_n(const Geo& g, const Band& b, const float2* Bt, int nf
     if (g.nx == NY && b.Wp == WP && std_band<NY>(b, static_band)) {
       const cudaError_t e = prep(k_col_t<NY, WP>, CC::SMEM);
       if (e != cudaSuccess) return e;
-      return launch_after(k_col_t<NY, WP>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt, nfs, scale, At);
+      return launch_after(k_col_t<NY, WP>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt,
+                          nfs, scale, At);
     }
   }
   const cudaError_t e = prep(k_col_t<NY>, CC::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_after(k_col_t<NY>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt, nfs, scale, At);
+  return launch_after(k_col_t<NY>, batch_grid(col_blocks(b, CC::C), nfs), CC::THREADS, CC::SMEM, st, g, b, Bt, nfs,
+                      scale, At);
 }
 cudaError_t launch_col_t(const Geo& g, const Band& b, const float2* Bt, int nfs, float scale, float2* At,
                          int static_band, cudaStream_t st) {
@@ -1349,7 +1337,8 @@ static cudaError_t probe_col_n(const Geo& g, const Band& ap, const float2* ex, c
   using CC = ProbeColCfg<NY>;
   const cudaError_t e = prep(k_probe_col<NY>, CC::SMEM);
   if (e != cudaSuccess) return e;
-  return launch_after(k_probe_col<NY>, batch_grid(col_blocks(ap, CC::C), P), CC::THREADS, CC::SMEM, st,  g, ap, ex, ey, chi, P, amp, Bpr);
+  return launch_after(k_probe_col<NY>, batch_grid(col_blocks(ap, CC::C), P), CC::THREADS, CC::SMEM, st, g, ap, ex,
+                      ey, chi, P, amp, Bpr);
 }
 cudaError_t launch_probe_col(const Geo& g, const Band& ap, const float2* ex, const float2* ey, const float2* chi,
                              int P, float amp, float2* Bpr, cudaStream_t st) {
@@ -1360,7 +1349,8 @@ template <int NX>
 static cudaError_t probe_row_n(const Geo& g, const Band& ap, const float2* Bpr, int P, float scale, float2* psi0,
                                cudaStream_t st) {
   using RC = ProbeRowCfg<NX>;
-  return launch_after(k_probe_row<NX>, batch_grid(g.ny / RC::G, P), RC::THREADS, RC::SMEM, st, g, ap, Bpr, P, scale, psi0);
+  return launch_after(k_probe_row<NX>, batch_grid(g.ny / RC::G, P), RC::THREADS, RC::SMEM, st, g, ap, Bpr, P, scale,
+                      psi0);
 }
 cudaError_t launch_probe_row(const Geo& g, const Band& ap, const float2* Bpr, int P, float scale, float2* psi0,
                              cudaStream_t st) {
@@ -1415,7 +1405,6 @@ static cudaError_t slice_row_n(const Geo& g, const Band& b, int first, int plane
   }
 #undef TACAW_SLICE_ROW_STD
 #undef TACAW_SLICE_ROW
-  return cudaGetLastError();
 }
 cudaError_t launch_slice_row(const Geo& g, const Band& b, int first, int plane, int tfused, const float2* Apsi,
                              const float2* psi0, const float2* t, int S, int s, int P, int nfc, float plane_amp,
@@ -1440,7 +1429,7 @@ static cudaError_t slice_col_n(const Geo& g, const Band& b, int last, const floa
   const dim3 grid = batch_grid(cb, (nw + wpb - 1) / wpb);
 #define TACAW_SLICE_COL(L, LOOP, ...)                                                                                 \
   do {                                                                                                                \
-    constexpr int SM = CC::SMEM + ((LOOP) ? NY * CC::C * (int)sizeof(float2) : 0);                                      \
+    constexpr int SM = CC::SMEM + ((LOOP) ? NY * CC::C * (int)sizeof(float2) : 0);                                     \
     cudaError_t e_ = prep(k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>, SM);                                   \
     if (e_ != cudaSuccess) return e_;                                                                                 \
     return launch_after(k_slice_col<NY, L, LOOP __VA_OPT__(, ) __VA_ARGS__>, grid, TH, SM, st, g, b, Bpsi, px, py,     \

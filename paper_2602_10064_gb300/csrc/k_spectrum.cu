@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(DP_BINS * DP_GROUPS)
 cudaError_t launch_detector_parts(const double* part, int64_t P, int64_t F, int64_t nparts, float* SI,
                                   cudaStream_t st) {
   if (P > 65535) return cudaErrorInvalidValue;
-  return launch_after(k_detector_parts, dim3((unsigned)((F + DP_BINS - 1) / DP_BINS), (unsigned)P), DP_BINS * DP_GROUPS, 0, st,  part, F, nparts, SI);
+  return launch_after(k_detector_parts, dim3((unsigned)((F + DP_BINS - 1) / DP_BINS), (unsigned)P),
+                      DP_BINS * DP_GROUPS, 0, st, part, F, nparts, SI);
 }
 
 // SI[p][m] = sum_j S[p][m][q_j], FP64 accumulation with a fixed reduction tree.

@@ -460,7 +460,8 @@ int spectrum_fft(tacaw_ctx* ctx, const float2* psi, int64_t P, int64_t F, const 
   const bool det = reduce == TACAW_REDUCE_DETECTOR;
   const int64_t nparts = det ? time_det_blocks(n, chirp, io.nsel) : 0;
   cudaError_t e;
-  if (det && (e = sc.get(&a.part, (size_t)P * nparts * F)) != cudaSuccess) return cuda_err(ctx, e, "detector partial sums");
+  if (det && (e = sc.get(&a.part, (size_t)P * nparts * F)) != cudaSuccess)
+    return cuda_err(ctx, e, "detector partial sums");
   const double pfq = (double)P * F * io.nsel;
   {
     ProfScope ps(ctx, "time_fft", sc.st, pfq * 8 + (det ? (double)P * nparts * F * 8 : pfq * 4),
@@ -497,7 +498,8 @@ int partial_fft(tacaw_ctx* ctx, const float2* psi, const float2* ref, int64_t P,
     const int rc = get_chirp(ctx, F, n, &a.chirp, &a.bhat);
     if (rc != TACAW_OK) return rc;
   }
-  ProfScope ps(ctx, "time_fft_partial", st, (double)P * nsel * 8 * (nf + F), (double)P * nsel * F * 5.0 * std::log2((double)std::max<int64_t>(F, 2)));
+  ProfScope ps(ctx, "time_fft_partial", st, (double)P * nsel * 8 * (nf + F),
+               (double)P * nsel * F * 5.0 * std::log2((double)std::max<int64_t>(F, 2)));
   const cudaError_t e = launch_time_fft(n, a, TIME_TILDE, chirp, st);
   return e == cudaSuccess ? TACAW_OK : cuda_err(ctx, e, "k_time_fft");
 }

@@ -31,8 +31,8 @@ struct FftPass {
   int r, ns;
 };
 constexpr FftPass kFftPasses[] = {
-    {4, 8},   {8, 8},    {4, 32},   {8, 32},  {16, 32}, {32, 32}, {4, 64},  {8, 64}, {4, 256}, {8, 16},  {16, 16},
-    {16, 64}, {16, 256}, {2, 256}, {8, 256}, {8, 12}, {8, 24}, {6, 64}, {12, 64}, {6, 24}, {8, 144}};
+    {4, 8},   {8, 8},    {4, 32},  {8, 32},  {16, 32}, {32, 32}, {4, 256}, {8, 16},  {16, 16},
+    {16, 256}, {2, 256}, {8, 256}, {8, 12},  {8, 24},  {6, 64},  {12, 64}, {6, 24}, {8, 144}};
 // Entries (float2) of the table of a pass.
 constexpr int pass_entries(int r, int ns) { return r == 2 ? ns : 2 * (r / 2) * ns; }
 // Start of its table, in float2 (all sizes are even: the pairs are 16-byte aligned); -1: no such pass.
@@ -133,9 +133,6 @@ __device__ __forceinline__ void pair_sub(float x, float mh, float ml, float& r, 
   two_sum(s, __fsub_rn(e, ml), r, re);
 }
 __device__ __forceinline__ int band_col_x(const Band& b, int nx, int c) { return c <= b.mb ? c : nx - (b.W - c); }
-__device__ __forceinline__ int band_x_col(const Band& b, int nx, int x) {
-  return x <= b.mb ? x : (x >= nx - b.mb ? x - nx + b.W : -1);
-}
 
 // Programmatic dependent launch: a kernel launched by launch_after may start once every block of the
 // kernel before it on the stream has started, and each of its threads waits here, before it touches
