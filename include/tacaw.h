@@ -138,8 +138,10 @@ int tacaw_bin_slices(tacaw_ctx* ctx, const tacaw_params* params, const float* po
  * V_s(r) = sum_k (2 pi a0 e / A) M(k) sum_{j in s} f_Zj(|k|) exp(2 pi i k.(r - r_j)), A = Lx Ly.
  * The structure factor is evaluated by spreading each atom onto the grid with an
  * exponential-of-semicircle kernel (width 12, beta 24) and deconvolving after the FFT.
- * pos: DEVICE float32 [nf][n_atoms][3] (A); Z: DEVICE int32 [n_atoms] (each Z must be in the
- * loaded table); V_out: DEVICE float32 [nf][S][ny][nx] (V*A).  The spread structure factor is
+ * pos: DEVICE float32 [nf][n_atoms][3] (A; an atom whose x or y is not finite adds nothing);
+ * Z: DEVICE int32 [n_atoms] (each Z must be in the loaded table: EINVAL, V_out untouched);
+ * V_out: DEVICE float32 [nf][S][ny][nx] (V*A), each slice's bits independent of the atoms of the
+ * others.  The call waits for the check of Z, not for its work.  The spread structure factor is
  * accurate only inside a band limit of at most 2/3 of Nyquist; EINVAL for bandlimit <= 0 or
  * > 2/3 (the same holds for tacaw_run). */
 int tacaw_build_potential(tacaw_ctx* ctx, const tacaw_params* params, const float* pos, const int32_t* Z,

@@ -8,7 +8,9 @@
 // result written once; the dense forms of the transform read it two or three times, write a
 // residual or split operands and do O(F) work per element where this does O(log F).  1024 frames x
 // 65536 q: 14.6 ms dense FP32, 0.27 ms here (3.0 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
-// 0.17 ms.  Bound by latency and the FP32 pipe.
+// 0.17 ms.  The image at 256 frames is bound by the FP32 pipe and latency (pipe 67% busy, 58% of the issue slots
+// by 22 warps, shared memory 39%, DRAM 35%), the forms of 1024 points by latency at the 8 warps that hold
+// them in registers (pipe 48%, issue 40%, DRAM 36%; chirp-z 46%, 49%, 13%).
 //
 // Mean and residual to FP64-class precision, as the dense forms have them: a column is summed as FP32
 // pairs (error-free two-sums, in the thread, over the lanes and over the warps), divided by F as a pair, and
@@ -109,9 +111,9 @@ constexpr int TIME_DET_TILES = 8;
 // The sums over the C columns of a CTA, C neighbouring lanes of a warp: n bins a lane as FP32 pairs.  In
 // each step two lanes O apart add theirs; while n is even each of the two keeps one half of the bins
 // (from e0 on), then both keep all and one of them writes.  In FP64 (three operations an element on a
-// pipe of two results a clock) these sums took a third of the pass at 256 frames; image of 32 probes, 256
-// frames 465 -> 435 us, ps an element at 32, 192, 512, 2048 frames 3.23 -> 2.56, 3.52 -> 2.67, 3.17 -> 2.73,
-// 5.88 -> 5.15.
+// pipe of two results a clock) these sums took a third of the pass at 256 frames.  Before the mean was summed
+// in pairs too: image of 32 probes, 256 frames 465 -> 435 us, ps an element at 32, 192, 512, 2048 frames
+// 3.23 -> 2.56, 3.52 -> 2.67, 3.17 -> 2.73, 5.88 -> 5.15.
 __host__ __device__ constexpr int kept_bins(int n, int c) { return c == 1 ? n : kept_bins(n % 2 ? n : n / 2, c / 2); }
 template <int n, int O>
 __device__ __forceinline__ void column_pairs(float* hi, float* lo, int c, int& e0, bool& writer) {
@@ -300,7 +302,8 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
       if (live) {
 #pragma unroll
         for (int e = 0; e < E; ++e) {
-          // FP32 pair: the exact errors of at most TIME_DET_TILES sums add up in lo
+          // FP32 pair: the exact errors of at most TIME_DET_TILES sums add up in lo, so that with the lanes'
+          // sums below a pair is off by less than 2^-43 of itself, 2^19 times less than the float returned
           float err;
           two_sum(hi[e], v[e].x * v[e].x + v[e].y * v[e].y, hi[e], err);
           lo[e] += err;
