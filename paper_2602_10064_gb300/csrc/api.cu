@@ -746,7 +746,8 @@ int bin_frames(tacaw_ctx* ctx, const tacaw_params& p, const float* pos, const in
 // A slice of a pair is rounded at the scale of the larger of the two.  A run takes that: its waves pass
 // both slices, and the error of their phases adds up to no more (exit waves of 54 slices of 1152 points
 // against 64 bits, three seeds: 7.7, 9.6, 8.2e-6 with pairs, 7.8, 9.6, 8.3e-6 without).  A V that is handed
-// out is held to its own scale: no pairs.
+// out is held to its own scale, without pairs (240 slices of 512 points 246 -> 373 us, 108 of 1152 0.77 ->
+// 1.31 ms).
 struct PotPlanes {
   const float2* Ap;
   int planes;           // in all
