@@ -1028,8 +1028,8 @@ struct RunPlan {
 };
 
 // The FP32 and the split-precision requests run as an FP32 FFT along the frames where there is a
-// length for them (every F up to 2048): 1024 frames x 65536 q 14.6 ms as a dense FP32 product, 0.27 ms
-// by FFT; 32 probes x 256 frames x 22880 q, spectrum image, 1.87 ms as BF16x3 products, 0.52 ms by
+// length for them (every F up to 2048): 1024 frames x 65536 q 14.6 ms as a dense FP32 product, 0.24 ms
+// by FFT; 32 probes x 256 frames x 22880 q, spectrum image, 1.87 ms as BF16x3 products, 0.46 ms by
 // FFT; the error against 64 bits falls from 1.2e-6 and 3.3e-6 to 1.3e-7 and 7e-8.  The single-product
 // requests, which ask for the tensor-core arithmetic itself, and longer trajectories take the dense forms.
 bool uses_time_fft(int32_t precision, int64_t F) {

@@ -7,18 +7,20 @@
 // psi~ itself (one process's share of a frame-sharded transform).  The stack is read once and the
 // result written once; the dense forms of the transform read it two or three times, write a
 // residual or split operands and do O(F) work per element where this does O(log F).  1024 frames x
-// 65536 q: 14.6 ms dense FP32, 0.27 ms here (3.0 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
-// 0.17 ms.  The image at 256 frames is bound by the FP32 pipe and latency (pipe 67% busy, 58% of the issue slots
-// by 22 warps, shared memory 39%, DRAM 35%), the forms of 1024 points by latency at the 8 warps that hold
-// them in registers (pipe 48%, issue 40%, DRAM 36%; chirp-z 46%, 49%, 13%).
+// 65536 q: 14.6 ms dense FP32, 0.24 ms here (3.3 TB/s); a partial transform of 256 of 512 frames: 2.14 ms,
+// 0.17 ms.  The image at 256 frames is bound by latency and the FP32 pipe (pipe 61% busy, 59% of the issue slots
+// by 22 warps, shared memory 44%, DRAM 40%), the forms of 1024 points by latency at the 8 warps that hold
+// them in registers (pipe 44%, issue 40%, DRAM 40%; chirp-z 44%, 49%, 14%).
 //
-// Mean and residual to FP64-class precision, as the dense forms have them: a column is summed as FP32
-// pairs (error-free two-sums, in the thread, over the lanes and over the warps), divided by F as a pair, and
-// r_n = psi_n - mean is formed exactly before it is rounded, once.  Columns that do not change give exactly
-// zero.  Plain FP32 sums of psi_n - psi_0 are faster (1024 frames x 65536 q 235 us, 266 now; image of 32
-// probes at 256 frames 435, 521; 501 frames 315, 346), but their error, the same in every frame, came
-// back F-fold in bin 0: up to 15 times the rounding of the sum itself in columns whose first frame stands
-// out.
+// Mean to FP64-class precision, as the dense forms have it: a column is summed as FP32 pairs (error-free
+// two-sums, in the thread, over the lanes and over the warps).  Every frame loses the mean rounded to float,
+// one subtraction with one rounding; what the rounded mean leaves of the column's sum, F times half a last
+// place at most, is the same in every frame, so it reaches bin 0 alone and is taken out of it there.  Columns
+// that do not change give exactly zero.  Plain FP32 sums of psi_n - psi_0 are faster (1024 frames x 65536 q
+// 235 us, 243 now; image of 32 probes at 256 frames 435, 463; 501 frames 315, 330), but round the residual
+// twice, and their own error came back F-fold in bin 0: up to 15 times the rounding of the sum itself in
+// columns whose first frame stands out.  Forming the residual exactly against a mean of two floats gave the
+// same and took longer (266, 521 and 346 us).
 //
 // Frame counts: the engine's own lengths directly; any other F up to 2048 by Bluestein's chirp-z
 // identity m n = (m^2 + n^2 - (m - n)^2) / 2, as a cyclic convolution of length M >= 2 F - 1 with a
@@ -42,8 +44,7 @@ enum TimeOut { TIME_S, TIME_DETECTOR, TIME_TILDE };
 // points S 3.21 -> 2.95, image 3.05 -> 2.85, chirp-z 7.64 -> 7.08; 512: S 4.99 -> 3.39, image 4.88 -> 3.14,
 // chirp-z 11.4 -> 8.0; 1024: S 7.02 -> 4.95, image 5.41 -> 4.42, chirp-z 13.0 -> 11.2; 2048: S 7.91 -> 7.54,
 // image 7.43 -> 5.87, chirp-z 19.8 -> 14.9; 4096: chirp-z 27.7 -> 16.9.  Now S, image, chirp-z S at 256 points
-// 3.05, 3.07, 7.18; 512: 3.79, 3.14, 8.52; 1024: 4.97, 4.38, 11.3; 2048: 7.53, 5.71, 14.8; two CTAs an SM of
-// 256 points in the image, 3.38, or six of half the columns, 3.19, lose to three.  16 columns are whole
+// 3.00, 2.73, 7.17; 512: 3.49, 2.86, 8.14; 1024: 4.95, 4.11, 10.7; 2048: 7.54, 5.46, 14.9.  16 columns are whole
 // 128-byte lines of the stack; more columns of the long transforms would leave one CTA per SM.
 struct TimeShape {
   int e, c, minb;
@@ -150,20 +151,13 @@ __device__ __forceinline__ void pair_add2(float2& h, float2& l, float2 xh, float
   two_sum2(h, xh, h, e);
   l = (l + xl) + e;
 }
-// (h + l) / F as (mh, ml): mh is the rounded product with 1 / F, whose remainder h - F mh is exact
-// (a few F units of mh's last place), and ml the quotient of what is left, corrected once, so that a
-// column of F equal frames has exactly that mean.
-__device__ __forceinline__ void pair_div2(float2 h, float2 l, float F, float inv, float2& mh, float2& ml) {
-  mh = inv * h;
-  const float2 rem = fma2(-F, mh, h) + l;
-  const float2 q = inv * rem;
-  ml = fma2(inv, fma2(-F, q, rem), q);
-}
-// x - (mh + ml), the first difference exact, so rounded once at the scale of the result
-__device__ __forceinline__ float2 pair_sub2(float2 x, float2 mh, float2 ml) {
-  float2 s, e;
-  two_sum2(x, make_float2(-mh.x, -mh.y), s, e);
-  return s + (e - ml);
+// The mean (h + l) / F rounded to float, and the rest of the sum, rest = h + l - F mean.  The remainder of
+// a rounded quotient, h - F q, is exact (a few F units of q's last place), so a column of F equal
+// frames has exactly that mean and no rest.
+__device__ __forceinline__ void pair_mean2(float2 h, float2 l, float F, float inv, float2& mean, float2& rest) {
+  const float2 q = inv * h;
+  mean = fma2(inv, fma2(-F, q, h) + l, q);
+  rest = fma2(-F, mean, h) + l;
 }
 
 template <int N, int OUT, bool BLUE>
@@ -240,7 +234,7 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
   for (int64_t tile = tile0; tile < tile1; ++tile) {
     const int64_t j = tile * C + c;
     const bool live = j < a.nsel;
-    float2 next[E], next0 = x0;
+    float2 next[E], next0 = x0, rest = make_float2(0.f, 0.f);
     if (TC::ASYNC) collect(v, x0);
     if (TC::PREFETCH && tile + 1 < tile1) load(next, next0, tile + 1);
     if constexpr (OUT == TIME_TILDE) {
@@ -277,11 +271,11 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
       }
 #pragma unroll
       for (int o = C; o < C * L; o <<= 1) pair_add2(hs, ls, shfl_xor2(hs, o), shfl_xor2(ls, o));
-      float2 mh, ml;
-      pair_div2(hs, ls, (float)F, 1.f / (float)F, mh, ml);
+      float2 mean;
+      pair_mean2(hs, ls, (float)F, 1.f / (float)F, mean, rest);
 #pragma unroll
       for (int e = 0; e < E; ++e)
-        v[e] = e < IN && (!BLUE || t + T * e < F) ? pair_sub2(v[e], mh, ml) : make_float2(0.f, 0.f);
+        v[e] = e < IN && (!BLUE || t + T * e < F) ? v[e] - mean : make_float2(0.f, 0.f);
     }
     // (both branches have passed a barrier after the slots were read)
     if (TC::ASYNC && tile + 1 < tile1) fetch(x0, tile + 1);
@@ -298,6 +292,7 @@ __global__ void __launch_bounds__(TimeCfg<N, OUT, BLUE>::THREADS, TimeCfg<N, OUT
     } else {
       fft<N, -1>(v, sm, idx, t, a.tw, sync);
     }
+    if (OUT != TIME_TILDE && t == 0) v[0] = v[0] - rest;
     if constexpr (OUT == TIME_DETECTOR) {
       if (live) {
 #pragma unroll
